@@ -220,6 +220,11 @@ cudaError_t launch_pack_slopes(const BlockDev* blocks, int nblk, int max_cols,
 cudaError_t launch_relayout(int dtype, const void* src, int na, int ns, const BlockDev* blocks,
                             int nblk, int max_pitch, void* dst, cudaStream_t st);
 
+// A narrow matrix in column blocks, row-major, into the order that launch_gemv reads (in
+// place; nothing to do for float32), with at most max_ctas CTAs per column block.
+cudaError_t launch_lane_order(int dtype, void* M, const BlockDev* blocks, int nblk, int rows, int max_pitch,
+                              int max_ctas, cudaStream_t st);
+
 // Per-row scaled quantisation (rtc_quantize_rows).
 cudaError_t launch_quantize(int dtype, int na, int ns, const float* M, size_t ld, void* codes,
                             float* scale, cudaStream_t st);

@@ -26,11 +26,14 @@ namespace rtc {
 size_t dtype_size(int dtype) { return dtype == RTC_F32 ? 4 : dtype == RTC_BF16 ? 2 : 1; }
 int elems_per_16B(int dtype) { return int(16 / dtype_size(dtype)); }
 
-__device__ __forceinline__ float warp_sum(float v) {
+// Sum over aligned groups of L lanes.
+template <int L>
+__device__ __forceinline__ float lane_sum(float v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = L / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+__device__ __forceinline__ float warp_sum(float v) { return lane_sum<32>(v); }
 
 // Programmatic dependent launch: a kernel lets the next one in its stream start
 // early (launch_dependents); the next one waits (wait) before it reads anything
@@ -558,10 +561,20 @@ cudaError_t launch_slopes(const SlopeCta* ctas, int cta0, int nctas, const WfsDe
 // a fixed xor-butterfly reduces the 32 lane sums.  The order of every sum is
 // fixed, so a block's partial does not depend on how the launch was split.
 // ---------------------------------------------------------------------------
+// Lanes to a row of an E4M3 matrix.  A block's row is short (MCAO: 69 vectors of 16
+// bytes), so 32 lanes leave its last step mostly empty (5 of 32 lanes); 16 lanes waste
+// less and a warp then works on two rows at a time per load of x.  MCAO MVM 99.9 us
+// before lane order, 88.7 us with 32 lanes, 81.6 us with 16, 106 us with 8 (one row per
+// lane: the loads of x are no longer shared); LTAO 63.0, 56.0, 54.8 and 67.1 us.
+#ifndef RTC_GEMV_E4M3_LANES
+#define RTC_GEMV_E4M3_LANES 16
+#endif
+constexpr int kLanesE4m3 = RTC_GEMV_E4M3_LANES;
+
 template <int DT> struct Elem;
-template <> struct Elem<RTC_F32> { static constexpr int kPer16 = 4; };
-template <> struct Elem<RTC_BF16> { static constexpr int kPer16 = 8; };
-template <> struct Elem<RTC_E4M3> { static constexpr int kPer16 = 16; };
+template <> struct Elem<RTC_F32> { static constexpr int kPer16 = 4, kLanes = 32; };
+template <> struct Elem<RTC_BF16> { static constexpr int kPer16 = 8, kLanes = 32; };
+template <> struct Elem<RTC_E4M3> { static constexpr int kPer16 = 16, kLanes = kLanesE4m3; };
 
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
     uint4 v;
@@ -574,9 +587,9 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
 
-// Vectors per lane of the single-block BF16 / E4M3 products without finalisation
-// (0: the MVM kernel).  E4M3 POLC, MCAO 26.6 -> 18.4 us, LTAO 20.4 -> 14.3 us (the
-// same with 4); BF16 unchanged at 2 or 4 (24.5 us: 235 CTAs over 152 SMs), so off.
+// Vectors per row of 32 lanes of the single-block BF16 / E4M3 products without
+// finalisation (0: the MVM kernel).  E4M3 POLC, MCAO 16.3 us, LTAO 14.2 us (the MVM
+// kernel: 26.6 and 20.4 us); BF16 unchanged at 2 (24.5 us), so off.
 #ifndef RTC_GEMV_BF16_U_DEEP
 #define RTC_GEMV_BF16_U_DEEP 0
 #endif
@@ -654,26 +667,39 @@ __device__ __forceinline__ float2 e4m3x2(uint32_t pair16) {
     return __half22float2(*reinterpret_cast<const __half2*>(&h));
 }
 
+// A vector's 16 products are summed by themselves, then added: 16 + the lane's vectors
+// roundings on the longest path in place of 16 times those vectors, which more than
+// makes up for the longer share of a row that each of fewer lanes has.
 template <typename A>
-__device__ __forceinline__ A dot_e4m3(const uint4& m, const float4* x, A acc) {
-    const uint32_t w[4] = {m.x, m.y, m.z, m.w};
+__device__ __forceinline__ A dot_e4m3(const uint4& m, const float4* x, int w, A acc) {
+    const uint32_t word[4] = {m.x, m.y, m.z, m.w};
+    A sum;
+    acc_zero(sum);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float4 xv = __ldg(x + k);
-        const float2 lo = e4m3x2(w[k] & 0xffffu);
-        const float2 hi = e4m3x2(w[k] >> 16);
-        acc = fma2(lo.x, lo.y, xv.x, xv.y, acc);
-        acc = fma2(hi.x, hi.y, xv.z, xv.w, acc);
+        const float4 xv = __ldg(x + k * w);
+        const float2 lo = e4m3x2(word[k] & 0xffffu);
+        const float2 hi = e4m3x2(word[k] >> 16);
+        sum = fma2(lo.x, lo.y, xv.x, xv.y, sum);
+        sum = fma2(hi.x, hi.y, xv.z, xv.w, sum);
     }
-    return acc;
+    return acc + sum;
 }
 
+// Lane order: the columns of an E4M3 row that the 16 bytes of a lane hold.  A row is
+// cut into groups of kL = kLanesE4m3 vectors, one per lane (the last group has w < kL),
+// and within a group a lane's k-th four codes are the columns 4 (k w + l) .. + 3, not
+// 4 (4 l + k) .. + 3.  So a load of x by the lanes of a row is contiguous (256 bytes;
+// with each lane's columns contiguous the lanes' loads are 64 bytes apart, and a warp's
+// load of x touches 16 128-byte lines in place of 2 or 4: MCAO MVM 99.9 -> 88.7 us with
+// 32 lanes to a row).  The matrix is put in this order once, when it is uploaded
+// (lane_order_kernel).
 template <int DT, typename A>
-__device__ __forceinline__ A dot16(const uint4& m, const float* x, int v, A acc) {
+__device__ __forceinline__ A dot16(const uint4& m, const float* x, int v, int l, int w, A acc) {
+    if constexpr (DT == RTC_E4M3) return dot_e4m3(m, reinterpret_cast<const float4*>(x) + (4 * v - 3 * l), w, acc);
     const float4* xp = reinterpret_cast<const float4*>(x) + v * (Elem<DT>::kPer16 / 4);
     if constexpr (DT == RTC_F32) return dot_f32(m, xp, acc);
     else if constexpr (DT == RTC_BF16) return dot_bf16(m, xp, acc);
-    else return dot_e4m3(m, xp, acc);
 }
 
 struct GemvArgs {
@@ -769,7 +795,8 @@ __device__ void finalise_tile(const FinaliseArgs& f, const float* __restrict__ p
 // kGated: a pre-enqueued chunk's MVM (the check of its mailbox costs the float32
 // variant two registers, so the other launches keep the kernels without it).
 // kGroup: consecutive column blocks per CTA (1: one block, the loop compiles away).
-template <int DT, int U, int RI, int RPW, bool kGated, int kGroup>
+// kLongRows: steps that lie wholly in the row get a loop of their own.
+template <int DT, int U, int RI, int RPW, bool kGated, int kGroup, bool kLongRows = false>
 __device__ __forceinline__ void gemv_body(const GemvArgs& a) {
     static_assert(RPW % RI == 0 && kFinRows % (kGemvWarps * RPW) == 0, "row tiling");
     __shared__ int s_last;
@@ -779,6 +806,10 @@ __device__ __forceinline__ void gemv_body(const GemvArgs& a) {
     const int g1 = kGroup == 1 ? g0 + 1 : min(g0 + kGroup, a.nb);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr size_t esz = 16 / Elem<DT>::kPer16;
+    // a warp works on RI rows at once, kL lanes to a row, kR rows and kU vectors of each in flight per lane
+    constexpr int kL = Elem<DT>::kLanes, kR = RI * kL / 32, kU = U * 32 / kL;
+    static_assert(kR >= 1, "lanes per row");
+    const int l = kL == 32 ? lane : lane % kL, rl = kL == 32 ? 0 : lane / kL * kR;
     const int r0 = tile * kGemvWarps * RPW;
     const int rbase = r0 + warp * RPW;
     BlockDev B = a.blocks[a.b0 + g0];                    // the first block's entry, before the wait
@@ -802,40 +833,57 @@ __device__ __forceinline__ void gemv_body(const GemvArgs& a) {
     const float* x = a.x + B.x_off;
 #pragma unroll 1
     for (int rr = 0; rr < RPW; rr += RI) {
-        const uint4* mrow[RI];
-        bool ok[RI];
-        typename AccOf<DT>::type acc[RI];
+        const uint4* mrow[kR];
+        bool ok[kR];
+        typename AccOf<DT>::type acc[kR];
 #pragma unroll
-        for (int i = 0; i < RI; ++i) {
-            const int r = rbase + rr + i;
-            ok[i] = r < a.na;
+        for (int i = 0; i < kR; ++i) {
+            const int r = rbase + rr + rl + i;
+            ok[i] = r < a.na;                          // E4M3 rows past the last read row 0 (not stored)
             mrow[i] = reinterpret_cast<const uint4*>(a.M + (size_t)(B.m_off + (long long)(ok[i] ? r : 0) * B.pitch) * esz);
             acc_zero(acc[i]);
         }
+        int vstart = l;
+        if constexpr (kLongRows) {                              // whole steps: nothing predicated, constant strides
 #pragma unroll 1
-        for (int v0 = lane; v0 < nvec; v0 += 32 * U) {
-            uint4 m[RI][U];
+            for (int v0 = l; v0 - l + kL * kU <= nvec; v0 += kL * kU) {
+                uint4 m[kR][kU];
 #pragma unroll
-            for (int i = 0; i < RI; ++i)
+                for (int i = 0; i < kR; ++i)
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int v = v0 + 32 * u;
-                    m[i][u] = (ok[i] && v < nvec) ? ld_stream(mrow[i] + v) : make_uint4(0u, 0u, 0u, 0u);
+                    for (int u = 0; u < kU; ++u) m[i][u] = ld_stream(mrow[i] + v0 + kL * u);
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+#pragma unroll
+                    for (int i = 0; i < kR; ++i) acc[i] = dot16<DT>(m[i][u], x, v0 + kL * u, l, kL, acc[i]);
+            }
+            vstart += nvec / (kL * kU) * (kL * kU);
+        }
+#pragma unroll 1
+        for (int v0 = vstart; v0 < nvec; v0 += kL * kU) {
+            uint4 m[kR][kU];
+#pragma unroll
+            for (int i = 0; i < kR; ++i)
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int v = v0 + kL * u;
+                    m[i][u] = ((DT == RTC_E4M3 || ok[i]) && v < nvec) ? ld_stream(mrow[i] + v) : make_uint4(0u, 0u, 0u, 0u);
                 }
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int v = v0 + 32 * u;
+            for (int u = 0; u < kU; ++u) {
+                const int v = v0 + kL * u;
                 if (v < nvec) {
+                    const int w = DT == RTC_E4M3 ? min(kL, nvec - (v - l)) : kL;      // vectors in the lanes' group
 #pragma unroll
-                    for (int i = 0; i < RI; ++i) acc[i] = dot16<DT>(m[i][u], x, v, acc[i]);
+                    for (int i = 0; i < kR; ++i) acc[i] = dot16<DT>(m[i][u], x, v, l, w, acc[i]);
                 }
             }
         }
 #pragma unroll
-        for (int i = 0; i < RI; ++i) {
-            const float t = warp_sum(acc_total(acc[i]));
-            const int r = rbase + rr + i;
-            if (lane == 0 && ok[i]) a.out[(long long)b * a.out_stride + r] = a.out_scale ? t * a.out_scale[r] : t;
+        for (int i = 0; i < kR; ++i) {
+            const float t = lane_sum<kL>(acc_total(acc[i]));
+            const int r = rbase + rr + rl + i;
+            if (l == 0 && ok[i]) a.out[(long long)b * a.out_stride + r] = a.out_scale ? t * a.out_scale[r] : t;
         }
     }
     }
@@ -876,28 +924,34 @@ __device__ __forceinline__ void gemv_body(const GemvArgs& a) {
     }
 }
 
+// Resident CTAs per SM that the MVM kernels' registers are held to.
+template <int DT> struct MinCtas { static constexpr int value = 8; };
+template <> struct MinCtas<RTC_BF16> { static constexpr int value = 4; };
+#ifndef RTC_GEMV_E4M3_CTAS
+#define RTC_GEMV_E4M3_CTAS 5
+#endif
+template <> struct MinCtas<RTC_E4M3> { static constexpr int value = RTC_GEMV_E4M3_CTAS; };
 template <int DT, int U, int RI, int RPW, bool kGated, int kGroup>
-__global__ void __launch_bounds__(kGemvWarps * 32) gemv_kernel(const __grid_constant__ GemvArgs a) {
+__global__ void __launch_bounds__(kGemvWarps * 32, DT == RTC_F32 ? 0 : MinCtas<DT>::value)
+    gemv_kernel(const __grid_constant__ GemvArgs a) {
     gemv_body<DT, U, RI, RPW, kGated, kGroup>(a);
 }
 
-// Several column blocks per CTA, held to the resident CTAs per SM of the one-block
-// kernel (the loop over blocks costs it registers otherwise).
-template <int DT> struct GroupedMinCtas { static constexpr int value = 8; };
-template <> struct GroupedMinCtas<RTC_BF16> { static constexpr int value = 4; };
-template <> struct GroupedMinCtas<RTC_E4M3> { static constexpr int value = 5; };
+// Several column blocks per CTA.
 template <int DT, int U, int RI, int RPW, bool kGated, int kGroup>
-__global__ void __launch_bounds__(kGemvWarps * 32, GroupedMinCtas<DT>::value)
+__global__ void __launch_bounds__(kGemvWarps * 32, MinCtas<DT>::value)
     gemv_kernel_grouped(const __grid_constant__ GemvArgs a) {
     gemv_body<DT, U, RI, RPW, kGated, kGroup>(a);
 }
 
 // A narrow format's single-block product without finalisation (the POLC product
 // P a, or D a): its few hundred CTAs hold under two per SM whatever their
-// registers, so each lane keeps more vectors in flight than the MVM kernels can.
+// registers, so each lane keeps more vectors in flight than the MVM kernels can, and
+// whole steps of its long rows run unpredicated (E4M3, MCAO: 20.4 -> 16.3 us).  In the
+// MVM kernels, whose rows are two steps long, that cost more than it gave (81.6 -> 90.8 us).
 template <int DT, int U, int RI, bool kGated>
 __global__ void __launch_bounds__(kGemvWarps * 32, 2) gemv_kernel_deep(const __grid_constant__ GemvArgs a) {
-    gemv_body<DT, U, RI, RI, kGated, 1>(a);
+    gemv_body<DT, U, RI, RI, kGated, 1, true>(a);
 }
 
 // One row per warp: the launches over a single column block (the POLC product, a
@@ -1110,6 +1164,43 @@ cudaError_t launch_relayout(int dtype, const void* src, int na, int ns, const Bl
             return launch_kernel(relayout_kernel<uint8_t>, grid, dim3(256), 0, st, (const uint8_t*)src, na, ns, blocks,
                                  (uint8_t*)dst);
     }
+}
+
+// Puts a row-major E4M3 matrix in column blocks into lane order (see dot16), in place:
+// kLanesE4m3 lanes take one group of as many vectors of a row at a time, read its words
+// of four codes coalesced in column order, and after all have read each writes its 16
+// bytes.
+__global__ void __launch_bounds__(256) lane_order_kernel(uint8_t* __restrict__ M, const BlockDev* __restrict__ blocks,
+                                                         int rows) {
+    constexpr int kL = kLanesE4m3, kPerWarp = 32 / kL;
+    const BlockDev B = blocks[blockIdx.y];
+    const int nvec = B.pitch / 16, groups = (nvec + kL - 1) / kL;
+    const int l = threadIdx.x % kL;
+    const long long total = (long long)rows * groups;
+    // all lanes of a warp take the same number of rounds (i0: its first group)
+    for (long long i0 = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * kPerWarp; i0 < total;
+         i0 += (long long)gridDim.x * 8 * kPerWarp) {
+        const long long i = i0 + (threadIdx.x & 31) / kL;
+        const int r = int(i / groups), g = int(i - (long long)r * groups);
+        const int w = i < total ? min(kL, nvec - kL * g) : 0;
+        uint4* const at = reinterpret_cast<uint4*>(M + B.m_off + (long long)r * B.pitch) + (long long)g * kL;
+        uint32_t u[4];
+        if (l < w) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) u[k] = reinterpret_cast<const uint32_t*>(at)[k * w + l];
+        }
+        __syncwarp();
+        if (l < w) at[l] = make_uint4(u[0], u[1], u[2], u[3]);
+    }
+}
+
+cudaError_t launch_lane_order(int dtype, void* M, const BlockDev* blocks, int nblk, int rows, int max_pitch,
+                              int max_ctas, cudaStream_t st) {
+    if (dtype != RTC_E4M3 || nblk <= 0 || rows <= 0 || max_pitch <= 0) return cudaSuccess;
+    constexpr int kPerCta = 256 / kLanesE4m3;
+    const long long groups = (long long)rows * ((max_pitch / 16 + kLanesE4m3 - 1) / kLanesE4m3);
+    const dim3 grid((unsigned)std::min<long long>((groups + kPerCta - 1) / kPerCta, max_ctas), nblk);
+    return launch_kernel(lane_order_kernel, grid, dim3(256), 0, st, static_cast<uint8_t*>(M), blocks, rows);
 }
 
 // One CTA per row: max |M_rj| (exact, order-free), the scale, then the codes.

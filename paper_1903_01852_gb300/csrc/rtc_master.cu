@@ -179,7 +179,8 @@ int create(const rtc_master_desc* d, rtc_master* m) {
         for (size_t r = 0; r < na; ++r)
             std::memcpy(rowed.data() + r * B.pitch * esz, static_cast<const unsigned char*>(P->P) + r * na * esz,
                         na * esz);
-        MCK(m, cudaMemcpy(m->d_P, rowed.data(), m->p_bytes, cudaMemcpyHostToDevice));
+        MCK(m, cudaMemcpyAsync(m->d_P, rowed.data(), m->p_bytes, cudaMemcpyHostToDevice, m->st));
+        MCK(m, launch_lane_order(m->p_dtype, m->d_P, m->d_pblock, 1, m->na, B.pitch, 4096, m->st));
         if (P->row_scale) {
             rc = malloc_dev(m, &m->d_pscale, na * 4);
             if (rc != RTC_OK) return rc;

@@ -434,6 +434,8 @@ int upload_matrix(rtc_loop* L, int dtype, const void* host, int rows, int cols, 
     }
     if (e == cudaSuccess && rc == RTC_OK && max_pitch > 0)
         e = launch_relayout(dtype, tmp, rows, cols, d_blocks, (int)blocks.size(), max_pitch, dst, L->st);
+    if (e == cudaSuccess && rc == RTC_OK && max_pitch > 0)
+        e = launch_lane_order(dtype, dst, d_blocks, (int)blocks.size(), rows, max_pitch, 4096, L->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(L->st);
     if (d_bad) cudaFree(d_bad);
     if (tmp) cudaFree(tmp);
@@ -1499,6 +1501,10 @@ int process_impl(rtc_loop* L, uint64_t id, const uint16_t* const* px, const size
     return status;
 }
 
+// CTAs of an update's reordering kernel over the whole matrix, few so that the frames
+// running meanwhile keep their bandwidth.
+constexpr int kUpdateCtas = 16;
+
 // Upload rows x width bytes from pageable host memory (row pitch spitch) into
 // device memory (row pitch dpitch >= width, the bytes past width written as
 // zeros) on the upload stream, through the loop's two page-locked staging
@@ -1510,6 +1516,8 @@ int process_impl(rtc_loop* L, uint64_t id, const uint16_t* const* px, const size
 int staged_upload(rtc_loop* L, void* dst, size_t dpitch, const void* src, size_t spitch, size_t width, size_t rows) {
     if (dpitch > kStageBytes) {
         CK(L, cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, cudaMemcpyHostToDevice, L->st_up));
+        if (dpitch > width)
+            CK(L, cudaMemset2DAsync(static_cast<unsigned char*>(dst) + width, dpitch, 0, dpitch - width, rows, L->st_up));
         return RTC_OK;
     }
     const size_t per = kStageBytes / dpitch;
@@ -1935,6 +1943,10 @@ int rtc_update(rtc_loop* L, const rtc_update_desc* d) {
                 TRY(staged_upload(L, static_cast<uint8_t*>(L->sh_M) + (size_t)B.m_off * esz, (size_t)B.pitch * esz,
                                   static_cast<const uint8_t*>(d->M) + (size_t)B.c0 * esz, (size_t)L->ns * esz,
                                   (size_t)B.ncols * esz, L->na));
+        int max_pitch = 0;
+        for (const BlockDev& B : L->blocks_h) max_pitch = std::max(max_pitch, B.pitch);
+        CK(L, launch_lane_order(L->m_dtype, L->sh_M, L->d_blocks, L->nblk, L->na, max_pitch,
+                                std::max(1, kUpdateCtas / std::max(1, L->nblk)), L->st_up));
         mask |= kUpdM;
     }
     if (d->M_scale) {
@@ -1945,6 +1957,7 @@ int rtc_update(rtc_loop* L, const rtc_update_desc* d) {
         const size_t pe = dtype_size(L->p_dtype);
         const size_t pitch = round_up((size_t)L->na, elems_per_16B(L->p_dtype));
         TRY(staged_upload(L, L->sh_P, pitch * pe, d->P, (size_t)L->na * pe, (size_t)L->na * pe, L->na));
+        CK(L, launch_lane_order(L->p_dtype, L->sh_P, L->d_pblock, 1, L->na, (int)pitch, kUpdateCtas, L->st_up));
         mask |= kUpdP;
     }
     if (d->P_scale) {
