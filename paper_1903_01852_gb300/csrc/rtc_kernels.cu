@@ -1203,40 +1203,146 @@ cudaError_t launch_lane_order(int dtype, void* M, const BlockDev* blocks, int nb
     return launch_kernel(lane_order_kernel, grid, dim3(256), 0, st, static_cast<uint8_t*>(M), blocks, rows);
 }
 
-// One CTA per row: max |M_rj| (exact, order-free), the scale, then the codes.
-__global__ void quantize_kernel(int dtype, int ns, const float* __restrict__ M, size_t ld, void* __restrict__ codes,
-                                float* __restrict__ scale) {
-    __shared__ float red[32];
-    const int r = blockIdx.x;
-    const float* row = M + (size_t)r * ld;
-    float m = 0.f;
-    for (int j = threadIdx.x; j < ns; j += blockDim.x) m = fmaxf(m, fabsf(row[j]));
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        m = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) red[0] = m;
-    }
-    __syncthreads();
-    float s = dtype == RTC_E4M3 ? __fdiv_rn(red[0], 448.0f) : red[0];
-    if (!(s > 0.f)) s = 1.0f;
-    if (threadIdx.x == 0) scale[r] = s;
-    if (dtype == RTC_BF16) {
-        __nv_bfloat16* out = static_cast<__nv_bfloat16*>(codes) + (size_t)r * ns;
-        for (int j = threadIdx.x; j < ns; j += blockDim.x) out[j] = __float2bfloat16_rn(__fdiv_rn(row[j], s));
+// Four quotients m / s as codes, the first in the low bits.  A code is that of the
+// quotient rounded to float32 (__fdiv_rn), which lies between m times lo and m times hi,
+// lo and hi being 1 / s less and more 2^-21 of itself: rounding to a code is monotone, so
+// where both products round to the same code, that is the quotient's.  Elsewhere (about
+// one element in 10^5 of a random E4M3 matrix, 10^3 of a BF16 one) it is divided out.  The
+// products are within 2^-23 of exact while they are normal numbers: `fast` says that s
+// allows it; an E4M3 code of a smaller product is zero whatever its error, a BF16 one is
+// divided out.
+template <int DT> struct Codes4;
+template <> struct Codes4<RTC_BF16> { using type = uint2; };
+template <> struct Codes4<RTC_E4M3> { using type = uint32_t; };
+
+template <int DT>
+__device__ __forceinline__ uint32_t code_pair(float a, float b) {
+    if constexpr (DT == RTC_BF16) {
+        const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+        return *reinterpret_cast<const uint32_t*>(&v);
     } else {
-        __nv_fp8_storage_t* out = static_cast<__nv_fp8_storage_t*>(codes) + (size_t)r * ns;
-        for (int j = threadIdx.x; j < ns; j += blockDim.x)
-            out[j] = __nv_cvt_float_to_fp8(__fdiv_rn(row[j], s), __NV_SATFINITE, __NV_E4M3);
+        return __nv_cvt_float2_to_fp8x2(make_float2(a, b), __NV_SATFINITE, __NV_E4M3);
     }
+}
+template <int DT>
+__device__ __forceinline__ typename Codes4<DT>::type join(uint32_t a, uint32_t b) {
+    if constexpr (DT == RTC_BF16) return make_uint2(a, b);
+    else return a | b << 16;
+}
+template <int DT>
+__device__ __forceinline__ typename Codes4<DT>::type codes4(const float4& m, float s, float lo, float hi, bool fast) {
+    const uint32_t a = code_pair<DT>(m.x * lo, m.y * lo), b = code_pair<DT>(m.z * lo, m.w * lo);
+    bool sure = fast && a == code_pair<DT>(m.x * hi, m.y * hi) && b == code_pair<DT>(m.z * hi, m.w * hi);
+    if constexpr (DT == RTC_BF16) {
+        auto small = [&](float v) { return fabsf(v * lo) < 1e-30f && v != 0.f; };
+        sure = sure && !(small(m.x) || small(m.y) || small(m.z) || small(m.w));
+    }
+    if (sure) return join<DT>(a, b);
+    return join<DT>(code_pair<DT>(__fdiv_rn(m.x, s), __fdiv_rn(m.y, s)),
+                    code_pair<DT>(__fdiv_rn(m.z, s), __fdiv_rn(m.w, s)));
+}
+
+__device__ __forceinline__ float abs_max4(float m, const float4& v) {
+    return fmaxf(fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+}
+
+// One CTA per row: max |M_rj| (exact, order-free), the scale, then the codes.  HBM
+// bounds it while the second reading of the row does not go there: at most two CTAs of a
+// long row run per SM, 304 rows of 222 KB (MCAO) or 68 MB against 126 MB of L2, and the
+// second reading goes backwards, so that it starts with what L1 still holds.  MCAO,
+// 7500 x 55608 to E4M3: 1387 us with one element a load, 256 threads and a division an
+// element, 339 us so (its 2.1 GB in one pass: 308 us); to BF16 429 us with the call (369 us).
+template <int DT, int kThreads, int kCtas>
+__global__ void __launch_bounds__(kThreads, kCtas)
+    quantize_kernel(int ns, const float* __restrict__ M, size_t ld, void* __restrict__ codes, float* __restrict__ scale) {
+    using Code = typename std::conditional<DT == RTC_BF16, uint16_t, uint8_t>::type;
+    using Four = typename Codes4<DT>::type;
+    constexpr int kU = kThreads == 1024 ? 2 : 4;          // vectors in flight (32 registers at 1024)
+    __shared__ float red[32];
+    const int r = blockIdx.x, t = threadIdx.x;
+    const float* const row = M + (size_t)r * ld;
+    Code* const out = static_cast<Code*>(codes) + (size_t)r * ns;
+    // the row: elements up to the first 16-byte boundary, whole vectors of four, the rest
+    const int head = min(ns, (int)((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) / 4);
+    const int nvec = (ns - head) / 4, tail = head + 4 * nvec;
+    const float4* const vec = reinterpret_cast<const float4*>(row + head);
+    const int rest = t < head ? t : tail + t - head;      // this thread's element outside the vectors, if < ns
+    const bool has_rest = t < head + ns - tail;
+    const float mr = has_rest ? row[rest] : 0.f;
+    float m = fabsf(mr);
+    m = fmaxf(0.f, m);                                    // a NaN counts as 0
+    int v = t;
+    for (; v + (kU - 1) * kThreads < nvec; v += kU * kThreads) {
+        float4 q[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) q[u] = vec[v + u * kThreads];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) m = abs_max4(m, q[u]);
+    }
+    for (; v < nvec; v += kThreads) m = abs_max4(m, vec[v]);
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((t & 31) == 0) red[t >> 5] = m;
+    __syncthreads();
+    m = (t & 31) < kThreads / 32 ? red[t & 31] : 0.f;
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    float s = DT == RTC_E4M3 ? __fdiv_rn(m, 448.0f) : m;
+    if (!(s > 0.f)) s = 1.0f;
+    if (t == 0) scale[r] = s;
+    const bool fast = s > 1e-30f && s < 1e30f;
+    const float inv = __fdiv_rn(1.0f, s), lo = inv * (1.0f - 0x1p-21f), hi = inv * (1.0f + 0x1p-21f);
+    const bool aligned = (reinterpret_cast<uintptr_t>(out + head) & (sizeof(Four) - 1)) == 0;
+    auto put = [&](int at, const float4& q) {
+        const Four c = codes4<DT>(q, s, lo, hi, fast);
+        Code* const o = out + head + 4 * at;
+        if (aligned) {
+            *reinterpret_cast<Four*>(o) = c;
+        } else {
+            Code one[4];
+            *reinterpret_cast<Four*>(one) = c;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) o[k] = one[k];
+        }
+    };
+    // backwards: the vectors after the last whole step, then the steps
+    const int steps = nvec / (kU * kThreads);
+    for (int at = steps * kU * kThreads + t; at < nvec; at += kThreads) put(at, vec[at]);
+    for (int k = steps - 1; k >= 0; --k) {
+        const int at = k * kU * kThreads + t;
+        float4 q[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) q[u] = vec[at + u * kThreads];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) put(at + u * kThreads, q[u]);
+    }
+    if (has_rest) {
+        const uint32_t c = code_pair<DT>(__fdiv_rn(mr, s), 0.f);
+        out[rest] = (Code)c;
+    }
+}
+
+// Threads a row by its length: enough CTAs run for the loads in flight, and few enough
+// that the rows being read stay in cache until their second reading.  200 M elements
+// to E4M3 in us (at most 12000 rows), 64 / 128 / 256 / 512 / 1024 threads, call included:
+// ns 1000: 19 23 31 52 81; 2000: 35 35 40 59 88; 6000: 84 69 72 83 123; 8608: 124 97 93
+// 113 156; 16000: 238 209 160 164 197; 20001: 257 234 184 170 216; 28000: 272 250 219 166
+// 193; 40000: 277 256 234 189 169.
+template <int DT>
+cudaError_t launch_quantize_t(int na, int ns, const float* M, size_t ld, void* codes, float* scale, cudaStream_t st) {
+    const auto launch = [&](auto kernel, int threads) {
+        return launch_kernel(kernel, dim3(na), dim3(threads), 0, st, ns, M, ld, codes, scale);
+    };
+    if (ns < 1536) return launch(quantize_kernel<DT, 64, 24>, 64);
+    if (ns < 7000) return launch(quantize_kernel<DT, 128, 12>, 128);
+    if (ns < 18000) return launch(quantize_kernel<DT, 256, 6>, 256);
+    if (ns < 34000) return launch(quantize_kernel<DT, 512, 3>, 512);
+    return launch(quantize_kernel<DT, 1024, 2>, 1024);
 }
 
 cudaError_t launch_quantize(int dtype, int na, int ns, const float* M, size_t ld, void* codes, float* scale,
                             cudaStream_t st) {
     if (na <= 0) return cudaSuccess;
-    return launch_kernel(quantize_kernel, dim3(na), dim3(256), 0, st, dtype, ns, M, ld, codes, scale);
+    if (dtype == RTC_BF16) return launch_quantize_t<RTC_BF16>(na, ns, M, ld, codes, scale, st);
+    return launch_quantize_t<RTC_E4M3>(na, ns, M, ld, codes, scale, st);
 }
 
 __global__ void check_finite_kernel(const float* __restrict__ x, size_t n, int* bad) {
