@@ -716,6 +716,7 @@ struct GemvArgs {
     FinaliseArgs fin;
     int prefetch_ctas;         // CTAs [0, prefetch_ctas) prefetch their matrix tile into L2 before waiting
     const int* gate_state;     // a pre-enqueued chunk's mailbox state: unless kChunkFilled, do nothing
+    bool whole;                // the MVM of a whole frame, finalised by a kernel of its own
     int group;                 // column blocks per CTA (consecutive, same row tile), >= 1
 };
 
@@ -792,11 +793,41 @@ __device__ void finalise_tile(const FinaliseArgs& f, const float* __restrict__ p
     }
 }
 
+// Finalises a tile; the last tile of the frame sets the completion word.
+template <bool kCounted>
+__device__ __forceinline__ void finish_tile(const FinaliseArgs& f, const float* __restrict__ partial, int na, int ft) {
+    finalise_tile(f, partial, na, ft);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (kCounted) f.counters[ft] = 0u;
+        if (f.done_flag) {
+            const int nfin = (na + kFinRows - 1) / kFinRows;
+            fence_acq_rel_sys();    // this tile's commands reach the host before the tile counts as done
+            if (atomicAdd(f.tiles_done, 1u) == (unsigned)(nfin - 1)) {
+                *f.tiles_done = 0u;
+                if (f.t_done) *f.t_done = global_time_ns();
+                fence_acq_rel_sys();
+                const unsigned long long seq = *reinterpret_cast<const volatile unsigned long long*>(f.seq);
+                *reinterpret_cast<volatile unsigned long long*>(f.done_flag) = seq;
+            }
+        }
+    }
+}
+
+// The finalisation of a whole frame as a kernel of its own, one CTA per tile, a
+// programmatic dependent of the MVM.
+__global__ void __launch_bounds__(kGemvWarps * 32)
+    finalise_kernel(const __grid_constant__ FinaliseArgs f, const float* __restrict__ partial, int na) {
+    pdl_wait();
+    pdl_trigger();
+    finish_tile<false>(f, partial, na, blockIdx.x);
+}
+
 // kGated: a pre-enqueued chunk's MVM (the check of its mailbox costs the float32
 // variant two registers, so the other launches keep the kernels without it).
 // kGroup: consecutive column blocks per CTA (1: one block, the loop compiles away).
 // kLongRows: steps that lie wholly in the row get a loop of their own.
-template <int DT, int U, int RI, int RPW, bool kGated, int kGroup, bool kLongRows = false>
+template <int DT, int U, int RI, int RPW, bool kGated, int kGroup, bool kLongRows = false, bool kFin = true>
 __device__ __forceinline__ void gemv_body(const GemvArgs& a) {
     static_assert(RPW % RI == 0 && kFinRows % (kGemvWarps * RPW) == 0, "row tiling");
     __shared__ int s_last;
@@ -887,7 +918,7 @@ __device__ __forceinline__ void gemv_body(const GemvArgs& a) {
         }
     }
     }
-    if (!a.fin.enabled) return;
+    if (!kFin || !a.fin.enabled) return;
     // Fused finalisation: the CTA that completes the last block of a row tile
     // (counted in rows, across launches of the same frame) finalises it.
     // Release/acquire through one thread: the barrier orders the CTA's partial
@@ -906,22 +937,7 @@ __device__ __forceinline__ void gemv_body(const GemvArgs& a) {
     }
     __syncthreads();
     if (!s_last) return;
-    finalise_tile(a.fin, a.out, a.na, ft);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        a.fin.counters[ft] = 0u;
-        if (a.fin.done_flag) {
-            const int nfin = (a.na + kFinRows - 1) / kFinRows;
-            fence_acq_rel_sys();    // this tile's commands reach the host before the tile counts as done
-            if (atomicAdd(a.fin.tiles_done, 1u) == (unsigned)(nfin - 1)) {
-                *a.fin.tiles_done = 0u;
-                if (a.fin.t_done) *a.fin.t_done = global_time_ns();
-                fence_acq_rel_sys();
-                const unsigned long long seq = *reinterpret_cast<const volatile unsigned long long*>(a.fin.seq);
-                *reinterpret_cast<volatile unsigned long long*>(a.fin.done_flag) = seq;
-            }
-        }
-    }
+    finish_tile<true>(a.fin, a.out, a.na, ft);
 }
 
 // Resident CTAs per SM that the MVM kernels' registers are held to.
@@ -960,6 +976,20 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) gemv_kernel_deep(const __g
 template <int DT, int U, int RI, bool kGated>
 __global__ void __launch_bounds__(kGemvWarps * 32, 8) gemv_kernel_1row(const __grid_constant__ GemvArgs a) {
     gemv_body<DT, U, RI, RI, kGated, 1>(a);
+}
+
+// The float32 MVM of a whole frame, finalised by a kernel of its own: the rows are read
+// once from HBM, so the loads in flight set the pace, and without the tail of the other
+// kernels (barrier, fence, ticket) a warp that is done frees its CTA's slot at once.
+// Eight vectors in flight per lane and five CTAs per SM (48 registers).  MVM alone, and
+// frame latency with the slope kernel overlapped, against gemv_kernel with its tail: ELT
+// SH (5316 x 8608) 40.5 -> 35.5 and 41.2 -> 36.6 us, ELT pyramid 50.8 -> 47.7 and 52.0 -> 45.0 us, MCAO 243.2 -> 242.3 and 251.2 -> 250.9 us.
+// With the tail: 42.6, 50.8, 247.5 us; nine vectors in flight 37.4, 49.8, 248.4 us; six
+// CTAs 35.5, 47.7, 244.3 us.
+constexpr int kWideU = 8;
+template <int RPW>
+__global__ void __launch_bounds__(kGemvWarps * 32, 5) gemv_kernel_wide(const __grid_constant__ GemvArgs a) {
+    gemv_body<RTC_F32, kWideU, 1, RPW, false, 1, false, false>(a);
 }
 
 // Telemetry entry of one frame: grid.y enumerates the recorded sections (one
@@ -1092,6 +1122,10 @@ cudaError_t launch_gemv_t(const GemvArgs& base, int nb, long long avg_row_bytes,
     if constexpr (kMaxGroup > 1)
         if (rpw >= 4 && a.group == kMaxGroup)
             return launch_maybe_pdl(gemv_kernel_grouped<DT, U, RI, (RI > 4 ? RI : 4), kG, kMaxGroup>, grid, a, pdl, st);
+    // rows of more vectors than the other float32 kernels keep in flight (4 x 32 of 16 bytes)
+    if constexpr (DT == RTC_F32 && !kG)
+        if (a.whole && avg_row_bytes > 2048)
+            return launch_maybe_pdl(rpw >= 4 ? gemv_kernel_wide<4> : gemv_kernel_wide<1>, grid, a, pdl, st);
     if (rpw >= 4) return launch_maybe_pdl(gemv_kernel<DT, U, RI, (RI > 4 ? RI : 4), kG, 1>, grid, a, pdl, st);
     if constexpr (!kNoRpw2)
         if (rpw >= 2) return launch_maybe_pdl(gemv_kernel<DT, U, RI, (RI > 2 ? RI : 2), kG, 1>, grid, a, pdl, st);
@@ -1099,27 +1133,53 @@ cudaError_t launch_gemv_t(const GemvArgs& base, int nb, long long avg_row_bytes,
     else return launch_maybe_pdl(gemv_kernel<DT, U, RI, RI, kG, 1>, grid, a, pdl, st);
 }
 
+template <bool kG>
+cudaError_t launch_gemv_dtype(int dtype, const GemvArgs& a, int nb, long long avg_row_bytes, bool pdl, cudaStream_t st) {
+    switch (dtype) {
+        case RTC_F32: return launch_gemv_t<RTC_F32, RTC_GEMV_F32_U, RTC_GEMV_F32_RI, kG>(a, nb, avg_row_bytes, pdl, st);
+        case RTC_BF16: return launch_gemv_t<RTC_BF16, RTC_GEMV_BF16_U, RTC_GEMV_BF16_RI, kG>(a, nb, avg_row_bytes, pdl, st);
+        case RTC_E4M3: return launch_gemv_t<RTC_E4M3, RTC_GEMV_E4M3_U, RTC_GEMV_E4M3_RI, kG>(a, nb, avg_row_bytes, pdl, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_finalise(const FinaliseArgs& fin, const float* partial, int na, cudaStream_t st) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((na + kFinRows - 1) / kFinRows);
+    cfg.blockDim = dim3(kGemvWarps * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, finalise_kernel, fin, partial, na);
+}
+
+// Bytes of a whole frame's matrix from which its finalisation is a kernel of its own.
+// Fused into the MVM's tail it costs every CTA a barrier, a fence and a ticket; as a
+// dependent kernel it costs a launch.  Frame period in us, fused / separate: float32
+// (with gemv_kernel_wide), 0.6 MB 21.5 / 22.2, 1 MB 23.6 / 22.6, 8 MB 24.7 / 23.5, 33 MB
+// 27.0 / 26.6; E4M3 3.5 MB 37.0 / 38.0, 14 MB 38.2 / 38.6, 57 MB 45.9 / 46.0, 417 MB
+// 116 / 112; BF16 8 MB 25.2 / 25.2, 834 MB 165 / 162.
+constexpr long long kSeparateMinF32 = 1LL << 20, kSeparateMinNarrow = 64LL << 20;
+
 cudaError_t launch_gemv(int dtype, const void* M, const BlockDev* blocks, int b0, int nb, int na, const float* x,
                         const float* out_scale, float* out, long long out_stride, const FinaliseArgs* fin,
                         long long avg_row_bytes, bool pdl, cudaStream_t st, const int* gate_state) {
     if (nb <= 0 || na <= 0) return cudaSuccess;
     GemvArgs a{static_cast<const uint8_t*>(M), blocks, b0, nb, 0, na, x, out_scale, out, out_stride, FinaliseArgs{}, 0,
-               gate_state, 1};
+               gate_state, false, 1};
     if (fin) a.fin = *fin;
-    if (gate_state) {
-        switch (dtype) {
-            case RTC_F32: return launch_gemv_t<RTC_F32, RTC_GEMV_F32_U, RTC_GEMV_F32_RI, true>(a, nb, avg_row_bytes, pdl, st);
-            case RTC_BF16: return launch_gemv_t<RTC_BF16, RTC_GEMV_BF16_U, RTC_GEMV_BF16_RI, true>(a, nb, avg_row_bytes, pdl, st);
-            case RTC_E4M3: return launch_gemv_t<RTC_E4M3, RTC_GEMV_E4M3_U, RTC_GEMV_E4M3_RI, true>(a, nb, avg_row_bytes, pdl, st);
-            default: return cudaErrorInvalidValue;
-        }
+    if (fin && fin->enabled && nb == fin->nblk && !gate_state &&
+        avg_row_bytes * na * nb >= (dtype == RTC_F32 ? kSeparateMinF32 : kSeparateMinNarrow)) {
+        a.fin = FinaliseArgs{};
+        a.whole = true;
+        const cudaError_t e = launch_gemv_dtype<false>(dtype, a, nb, avg_row_bytes, pdl, st);
+        return e != cudaSuccess ? e : launch_finalise(*fin, out, na, st);
     }
-    switch (dtype) {
-        case RTC_F32: return launch_gemv_t<RTC_F32, RTC_GEMV_F32_U, RTC_GEMV_F32_RI, false>(a, nb, avg_row_bytes, pdl, st);
-        case RTC_BF16: return launch_gemv_t<RTC_BF16, RTC_GEMV_BF16_U, RTC_GEMV_BF16_RI, false>(a, nb, avg_row_bytes, pdl, st);
-        case RTC_E4M3: return launch_gemv_t<RTC_E4M3, RTC_GEMV_E4M3_U, RTC_GEMV_E4M3_RI, false>(a, nb, avg_row_bytes, pdl, st);
-        default: return cudaErrorInvalidValue;
-    }
+    if (gate_state) return launch_gemv_dtype<true>(dtype, a, nb, avg_row_bytes, pdl, st);
+    return launch_gemv_dtype<false>(dtype, a, nb, avg_row_bytes, pdl, st);
 }
 
 __global__ void pack_slopes_kernel(const BlockDev* __restrict__ blocks, const float* __restrict__ s_pad,
