@@ -587,15 +587,6 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
 __device__ __forceinline__ float bf_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
 
-// Vectors per row of 32 lanes of the single-block BF16 / E4M3 products without
-// finalisation (0: the MVM kernel).  E4M3 POLC, MCAO 16.3 us, LTAO 14.2 us (the MVM
-// kernel: 26.6 and 20.4 us); BF16 unchanged at 2 (24.5 us), so off.
-#ifndef RTC_GEMV_BF16_U_DEEP
-#define RTC_GEMV_BF16_U_DEEP 0
-#endif
-#ifndef RTC_GEMV_E4M3_U_DEEP
-#define RTC_GEMV_E4M3_U_DEEP 2
-#endif
 #ifndef RTC_GEMV_GROUP_MIN_WAVES
 #define RTC_GEMV_GROUP_MIN_WAVES 2 // waves of 8 CTAs per SM a grouped launch keeps at least
 #endif
@@ -960,15 +951,28 @@ __global__ void __launch_bounds__(kGemvWarps * 32, MinCtas<DT>::value)
     gemv_body<DT, U, RI, RPW, kGated, kGroup>(a);
 }
 
-// A narrow format's single-block product without finalisation (the POLC product
-// P a, or D a): its few hundred CTAs hold under two per SM whatever their
+// A narrow format's launch of few CTAs (the POLC product P a; an MVM of few or long
+// column blocks, a row chunk's): they hold under two or so per SM whatever their
 // registers, so each lane keeps more vectors in flight than the MVM kernels can, and
-// whole steps of its long rows run unpredicated (E4M3, MCAO: 20.4 -> 16.3 us).  In the
-// MVM kernels, whose rows are two steps long, that cost more than it gave (81.6 -> 90.8 us).
+// whole steps of its rows run unpredicated (E4M3 POLC, MCAO: 20.4 -> 16.3 us; in the MVM
+// kernels, whose rows are two steps long, that cost more than it gave, 81.6 -> 90.8 us).
+// Up to 152 CTAs of four rows per warp, two rows per warp make twice as many.
 template <int DT, int U, int RI, bool kGated>
 __global__ void __launch_bounds__(kGemvWarps * 32, 2) gemv_kernel_deep(const __grid_constant__ GemvArgs a) {
     gemv_body<DT, U, RI, RI, kGated, 1, true>(a);
 }
+
+// Which launches take it, and the vectors per row of 32 lanes.  Frame period in us of
+// an SH sensor of n x n, column blocks, rows: n / blocks / rows (CTAs), MVM kernel / deep,
+// E4M3: 71/1/1065 (34) 41.1 / 27.0 (two rows; 29.7 with four), 42/1/1539 (49) 27.8 / 23.5,
+// 74/1/5316 (167) 44.0 / 31.8, 74/8/1000 (256) 26.1 / 24.6; rows of 4.3 KB, 74/2/5316
+// (334) 34.8 / 32.8; but rows of 1 KB, 74/8/2000 (504) 26.6 / 27.3.
+// BF16: 71/1/1065 34.7 / 27.2 (29.3), 42/1/1539 25.9 / 23.5, 74/1/5316 39.4 / 36.1,
+// 74/8/1000 25.7 / 25.3, but 74/2/5316 33.9 / 36.1, 74/8/2000 26.9 / 28.0.
+// POLC products: BF16 MCAO (235 CTAs) 24.5 / 22.5 us, LTAO (167) 18.3 / 16.2; E4M3 26.6 /
+// 16.3 and 20.4 / 13.2.
+template <int DT> struct Deep { static constexpr int kU = 3, kMaxCtas = 304, kLongRowFactor = 1; };
+template <> struct Deep<RTC_E4M3> { static constexpr int kU = 2, kMaxCtas = 304, kLongRowFactor = 2; };
 
 // One row per warp: the launches over a single column block (the POLC product, a
 // row chunk's block) have about a thousand CTAs, and at <= 32 registers all of
@@ -1100,12 +1104,18 @@ cudaError_t launch_gemv_t(const GemvArgs& base, int nb, long long avg_row_bytes,
     if (kNoRpw2 && rpw == 2) rpw = 1;
     GemvArgs a = base;
     a.tiles = (na + kGemvWarps * rpw - 1) / (kGemvWarps * rpw);
-    constexpr int kUDeep = DT == RTC_BF16 ? RTC_GEMV_BF16_U_DEEP : DT == RTC_E4M3 ? RTC_GEMV_E4M3_U_DEEP : 0;
-    if constexpr (kUDeep > 0 && RI == 4) {
-        if (!a.fin.enabled && nb == 1 && rpw == RI && a.tiles <= 2 * 152) {
-            const long long tile_bytes = std::max(1LL, avg_row_bytes * kGemvWarps * rpw);
-            a.prefetch_ctas = pdl ? (int)std::min<long long>(a.tiles, (96LL << 20) / tile_bytes) : 0;
-            return launch_maybe_pdl(gemv_kernel_deep<DT, kUDeep, RI, kG>, dim3((unsigned)a.tiles), a, pdl, st);
+    // few CTAs: deep kernels (see Deep)
+    if constexpr (DT != RTC_F32 && RI == 4) {
+        const long long ctas = (long long)a.tiles * nb;
+        if (rpw == RI && ctas <= Deep<DT>::kMaxCtas * (avg_row_bytes >= 2048 ? Deep<DT>::kLongRowFactor : 1)) {
+            const int rows = ctas <= 152 ? 2 : RI;
+            a.tiles = (na + kGemvWarps * rows - 1) / (kGemvWarps * rows);
+            const long long tile_bytes = std::max(1LL, avg_row_bytes * kGemvWarps * rows);
+            const dim3 grid((unsigned)(a.tiles * nb));
+            a.prefetch_ctas = pdl ? (int)std::min<long long>(grid.x, (96LL << 20) / tile_bytes) : 0;
+            constexpr int kU = Deep<DT>::kU;
+            return launch_maybe_pdl(rows == RI ? gemv_kernel_deep<DT, kU, RI, kG> : gemv_kernel_deep<DT, kU, 2, kG>, grid, a,
+                                    pdl, st);
         }
     }
     // consecutive column blocks per CTA, as many as keep that many waves
