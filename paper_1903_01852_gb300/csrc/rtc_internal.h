@@ -122,7 +122,7 @@ struct FramePtrs {
 // One reconstruction column block, stored as a dense [na][pitch] sub-matrix.
 struct BlockDev {
     long long m_off;          // element offset of the sub-matrix
-    int x_off;                // padded input-vector index of the block's first column
+    int x_off;                // padded input-vector index of the block's first column (a multiple of 32)
     int ncols;                // true columns
     int pitch;                // stored columns (multiple of 16 bytes / element size)
     int c0;                   // compact index of the block's first column
@@ -193,11 +193,13 @@ cudaError_t launch_normalise(const int2* items, int item0, int nitems, int max_p
 // (nwfs entries, host memory) travels in the kernel parameters.  host_px: the
 // variant that keeps all of a thread's pixel rows in flight, for small launches
 // that read pixels in place from page-locked host memory.  Each slope is
-// (measured - ref) + pol, with ref and pol (compact slope order) optional.
+// (measured - ref) + pol, with ref and pol (compact slope order) optional.  beside:
+// launched as a programmatic dependent of the stream's last kernel, which must be one of
+// the same frame on other slope rows; it starts beside that kernel and ends after it.
 cudaError_t launch_slopes(const SlopeCta* ctas, int cta0, int nctas, const WfsDev* wfs, int nwfs,
                           const FramePtrs& fp, bool host_px, const uint16_t* xlist, const float* ref,
                           const float* pol, float* s_pad, float* pscr, unsigned* counters, int smem_bytes,
-                          cudaStream_t st, const ChunkGate* gate = nullptr);
+                          cudaStream_t st, const ChunkGate* gate = nullptr, bool beside = false);
 
 // GEMV over blocks [b0, b0 + nb): out[b * out_stride + r] = sum_j M_b[r][j] x[x_off_b + j],
 // times out_scale[r] when out_scale is not NULL; with fin, the CTA completing the

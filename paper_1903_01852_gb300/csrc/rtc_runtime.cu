@@ -566,7 +566,9 @@ int create_impl(const rtc_geometry* G, const rtc_calib* C, const rtc_cmat* M, co
             B.ncols = local;
             B.pitch = (int)round_up((size_t)local, (size_t)V);
             compact += local;
-            x_off += B.pitch;
+            // a 128-byte line of the slope vector belongs to one block: chunks and cameras write theirs
+            // while the MVM of another block reads
+            x_off += (int)round_up((size_t)B.pitch, 32);
             m_off += (long long)L->na * B.pitch;
             L->blk_row_end.push_back(r1);
             L->blocks_h.push_back(B);
@@ -1165,11 +1167,11 @@ FinaliseArgs fin_args(rtc_loop* L) {
 // the slope kernel variant with all of a thread's pixel rows in flight.
 // gate: a pre-enqueued chunk's mailbox (its CTAs wait on it for the pixel address).
 int slopes_rows(rtc_loop* L, int r0, int r1, const FramePtrs& fp, bool host_px, cudaStream_t st,
-                const ChunkGate* gate = nullptr) {
+                const ChunkGate* gate = nullptr, bool beside = false) {
     const int p0 = L->part_start[r0], p1 = L->part_start[r1];
     const float* pol = L->explicit_polc ? L->d_u : nullptr;
     CK(L, launch_slopes(L->d_ctas, p0, p1 - p0, L->wfs_host.data(), L->nwfs, fp, host_px, L->d_xlist, L->d_ref, pol,
-                        L->d_s, L->d_pscr, L->d_row_cnt, L->smem_bytes, st, gate));
+                        L->d_s, L->d_pscr, L->d_row_cnt, L->smem_bytes, st, gate, beside));
     // globally normalised pyramids whose rows all ran here (they are never split across launches)
     int i0 = -1, i1 = -1;
     for (int k = 0; k < L->nwfs; ++k)
@@ -1375,7 +1377,10 @@ int submit_impl(rtc_loop* L, const rtc_chunk* c) {
         L->rows_in[k] = c->row_end;
         const bool slopes_launched = upto > done;
         if (slopes_launched) {
-            TRY(slopes_rows(L, r0 + done, r0 + upto, fp, in_place && host_px, sk));
+            // a camera's later chunk, read in place: its slopes run beside the MVM of the chunk before (the
+            // stream's last kernel is this frame's; with timing or pre-enqueued chunks events lie between)
+            const bool beside = done > 0 && in_place && !L->timing && !L->prelaunch;
+            TRY(slopes_rows(L, r0 + done, r0 + upto, fp, in_place && host_px, sk, nullptr, beside));
             L->rows_done[k] = upto;
         }
         if (last && L->stage_timing) CK(L, cudaEventRecord(s.ev_slopes, sk));
