@@ -1110,34 +1110,31 @@ cudaError_t launch_gemv_t(const GemvArgs& base, int nb, long long avg_row_bytes,
     if (kNoRpw2 && rpw == 2) rpw = 1;
     GemvArgs a = base;
     a.tiles = (na + kGemvWarps * rpw - 1) / (kGemvWarps * rpw);
+    const auto fill = [&](int rows, int group) {            // the grid, and the prefetch of its first tiles
+        a.tiles = (na + kGemvWarps * rows - 1) / (kGemvWarps * rows);
+        a.group = group;
+        const dim3 grid((unsigned)(a.tiles * ((nb + group - 1) / group)));
+        // prefetch while waiting for the producer: about 96 MB, below the L2 size
+        const long long tile_bytes = std::max(1LL, avg_row_bytes * kGemvWarps * rows * group);
+        a.prefetch_ctas = pdl ? (int)std::min<long long>(grid.x, (96LL << 20) / tile_bytes) : 0;
+        return grid;
+    };
+    // consecutive column blocks per CTA, if that keeps enough CTAs
+    constexpr int kMaxGroup = DT == RTC_F32 ? RTC_GEMV_GROUP_F32 : DT == RTC_BF16 ? RTC_GEMV_GROUP_BF16 : RTC_GEMV_GROUP_E4M3;
+    if constexpr (kMaxGroup > 1)
+        if (rpw >= 4 && (long long)a.tiles * ((nb + kMaxGroup - 1) / kMaxGroup) >= RTC_GEMV_GROUP_MIN_WAVES * 8LL * 152)
+            return launch_maybe_pdl(gemv_kernel_grouped<DT, U, RI, (RI > 4 ? RI : 4), kG, kMaxGroup>, fill(rpw, kMaxGroup), a,
+                                    pdl, st);
     // few CTAs: deep kernels (see Deep)
     if constexpr (DT != RTC_F32 && RI == 4) {
         const long long ctas = (long long)a.tiles * nb;
         if (rpw == RI && ctas <= Deep<DT>::kMaxCtas * (avg_row_bytes >= 2048 ? Deep<DT>::kLongRowFactor : 1)) {
-            const int rows = ctas <= 152 ? 2 : RI;
-            a.tiles = (na + kGemvWarps * rows - 1) / (kGemvWarps * rows);
-            const long long tile_bytes = std::max(1LL, avg_row_bytes * kGemvWarps * rows);
-            const dim3 grid((unsigned)(a.tiles * nb));
-            a.prefetch_ctas = pdl ? (int)std::min<long long>(grid.x, (96LL << 20) / tile_bytes) : 0;
             constexpr int kU = Deep<DT>::kU;
-            return launch_maybe_pdl(rows == RI ? gemv_kernel_deep<DT, kU, RI, kG> : gemv_kernel_deep<DT, kU, 2, kG>, grid, a,
-                                    pdl, st);
+            if (ctas <= 152) return launch_maybe_pdl(gemv_kernel_deep<DT, kU, 2, kG>, fill(2, 1), a, pdl, st);
+            return launch_maybe_pdl(gemv_kernel_deep<DT, kU, RI, kG>, fill(RI, 1), a, pdl, st);
         }
     }
-    // consecutive column blocks per CTA, as many as keep that many waves
-    constexpr int kMaxGroup = DT == RTC_F32 ? RTC_GEMV_GROUP_F32 : DT == RTC_BF16 ? RTC_GEMV_GROUP_BF16 : RTC_GEMV_GROUP_E4M3;
-    // (one grouped instance, kMaxGroup, used when four rows per warp keep that many waves with it)
-    a.group = 1;
-    if (kMaxGroup > 1 && rpw >= 4 &&
-        (long long)a.tiles * ((nb + kMaxGroup - 1) / kMaxGroup) >= RTC_GEMV_GROUP_MIN_WAVES * 8LL * 152)
-        a.group = kMaxGroup;
-    const dim3 grid((unsigned)(a.tiles * ((nb + a.group - 1) / a.group)));
-    // prefetch while waiting for the producer: about 96 MB, below the L2 size
-    const long long tile_bytes = std::max(1LL, avg_row_bytes * kGemvWarps * rpw * a.group);
-    a.prefetch_ctas = pdl ? (int)std::min<long long>(grid.x, (96LL << 20) / tile_bytes) : 0;
-    if constexpr (kMaxGroup > 1)
-        if (rpw >= 4 && a.group == kMaxGroup)
-            return launch_maybe_pdl(gemv_kernel_grouped<DT, U, RI, (RI > 4 ? RI : 4), kG, kMaxGroup>, grid, a, pdl, st);
+    const dim3 grid = fill(rpw, 1);
     // rows of more vectors than the other float32 kernels keep in flight (4 x 32 of 16 bytes)
     if constexpr (DT == RTC_F32 && !kG)
         if (a.whole && avg_row_bytes > 2048)
