@@ -217,6 +217,14 @@ def _pitch(x):
     return x.strides[0]
 
 
+_one_float = C.c_float * 1
+
+
+def _own(a):
+    """A new float32 array as a float pointer argument (a fifth of the time of ctypes.data_as)."""
+    return _one_float.from_buffer(a) if a.size else a.ctypes.data_as(f32p)
+
+
 class _Described:
     """The C structs of one loop description, and the arrays they point into."""
 
@@ -313,7 +321,6 @@ class Loop:
             self._h = C.c_void_p(_handle)
         inf = self.info()
         self.ns = inf["ns"]
-        self._cmd = np.empty(self.na, np.float32)
 
     # -- lifetime ---------------------------------------------------------
     def close(self):
@@ -373,8 +380,11 @@ class Loop:
     def process_frame(self, frame_id, dev_frames):
         """Whole frame from device-resident uint16 tensors (one per WFS)."""
         n = len(dev_frames)
-        px = (C.c_void_p * n)(*[t.data_ptr() for t in dev_frames])
-        pitch = (C.c_size_t * n)(*[t.stride(0) * t.element_size() for t in dev_frames])
+        px = (C.c_void_p * n)()
+        pitch = (C.c_size_t * n)()
+        for k, t in enumerate(dev_frames):
+            px[k] = t.data_ptr()
+            pitch[k] = t.stride(0) * t.element_size()
         return _check(lib.rtc_process_frame(self._h, frame_id, px, pitch), self._h, allow=(RTC_EDROPPED,))
 
     def next_frame_buffers(self):
@@ -395,9 +405,13 @@ class Loop:
         return _check(lib.rtc_submit_frame_graph(self._h, frame_id), self._h, allow=(RTC_EDROPPED,))
 
     def get_commands(self, timeout_us=-1, out=None):
-        out = self._cmd.copy() if out is None else out
+        if out is None:
+            out = np.empty(self.na, np.float32)
+            ptr = _own(out)
+        else:
+            ptr = out.ctypes.data_as(f32p)
         fid = C.c_uint64()
-        rc = lib.rtc_get_commands(self._h, out.ctypes.data_as(f32p), self.na, C.byref(fid), int(timeout_us))
+        rc = lib.rtc_get_commands(self._h, ptr, self.na, C.byref(fid), int(timeout_us))
         if rc == RTC_ETIMEDOUT:
             raise TimeoutError(_err(self._h))
         _check(rc, self._h)
@@ -406,8 +420,7 @@ class Loop:
     def get_telemetry(self, frame_id, timeout_us=-1):
         s = np.empty(self.ns, np.float32)
         a = np.empty(self.na, np.float32)
-        _check(lib.rtc_get_telemetry(self._h, frame_id, s.ctypes.data_as(f32p), self.ns,
-                                     a.ctypes.data_as(f32p), self.na, int(timeout_us)), self._h)
+        _check(lib.rtc_get_telemetry(self._h, frame_id, _own(s), self.ns, _own(a), self.na, int(timeout_us)), self._h)
         return s, a
 
     def telemetry_read(self, timeout_us=-1, slopes=True, cmds=True, partials=False):
