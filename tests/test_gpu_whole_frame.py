@@ -57,3 +57,32 @@ def test_whole_frames_equal_chunked_ones_bitwise(rtc, nsub, na, nblocks):
         ref = OracleLoop(cfg)
         for a, f in zip(got["whole"], frames):
             assert rel(a, ref.step(f)[1]) <= TOL_F32
+
+
+@pytest.mark.parametrize("fmt, nsub, na, nblocks", [("f32", 24, 200, 3), ("f32", 40, 1001, 4), ("bf16", 40, 2500, 4),
+                                                    ("e4m3", 40, 2500, 8)])
+def test_frames_in_a_row_start_beside_the_polc_product(rtc, fmt, nsub, na, nblocks):
+    # With an implicit POLC a frame's slopes run beside the POLC product of the frame before.  Frames submitted
+    # three at a time before their commands are read, with and without slope telemetry, against a loop whose
+    # timing events keep them apart.
+    pytest.importorskip("torch")
+    from oracle import quantize_rows
+    cfg = config(nsub, na, nblocks, clip=(-0.3, 0.3))
+    if fmt != "f32":
+        (m, ms), (p, ps) = quantize_rows(cfg["M"], fmt), quantize_rows(cfg["P"], fmt)
+        cfg.update(M=m, M_scale=ms, M_dtype=fmt, P=p, P_scale=ps, P_dtype=fmt)
+    frames = [device_frames(f) for f in synth.draw_frames(cfg, 5, seed=702)]
+    want = []
+    with rtc.Loop(cfg, timing=True) as loop:
+        for k in range(30):
+            loop.process_frame(k + 1, frames[k % 5])
+            want.append(loop.get_commands(timeout_us=WAIT_US)[1])
+    for telemetry in (False, True):
+        with rtc.Loop(cfg, telemetry=telemetry) as loop:
+            for k in range(0, 30, 3):
+                for j in range(3):
+                    loop.process_frame(k + j + 1, frames[(k + j) % 5])
+                for j in range(3):
+                    fid, a = loop.get_commands(timeout_us=WAIT_US)
+                    assert fid == k + j + 1 and np.array_equal(a, want[k + j]), (telemetry, k + j)
+            assert loop.check_guards() == 0
