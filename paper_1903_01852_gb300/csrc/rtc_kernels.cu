@@ -997,17 +997,22 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 8) gemv_kernel_1row(const __g
     gemv_body<DT, U, RI, RI, kGated, 1>(a);
 }
 
-// The float32 MVM of a whole frame, finalised by a kernel of its own: the rows are read
-// once from HBM, so the loads in flight set the pace, and without the tail of the other
-// kernels (barrier, fence, ticket) a warp that is done frees its CTA's slot at once.
-// Eight vectors in flight per lane and five CTAs per SM (48 registers).  MVM alone, and
-// frame latency with the slope kernel overlapped, against gemv_kernel with its tail: ELT
-// SH (5316 x 8608) 40.5 -> 35.5 and 41.2 -> 36.6 us, ELT pyramid 50.8 -> 47.7 and 52.0 -> 45.0 us, MCAO 243.2 -> 242.3 and 251.2 -> 250.9 us.
-// With the tail: 42.6, 50.8, 247.5 us; nine vectors in flight 37.4, 49.8, 248.4 us; six
-// CTAs 35.5, 47.7, 244.3 us.
-constexpr int kWideU = 8;
+// The float32 MVM of a whole frame, finalised by a kernel of its own, and float32
+// products of one wave (a POLC of up to 6080 actuators).  The rows are read once from
+// HBM, so the loads in flight set the pace, and without the tail of the other kernels
+// (barrier, fence, ticket) a warp that is done frees its CTA's slot at once.  Eight
+// vectors in flight per lane and five CTAs per SM (48 registers).  MVM alone, and frame
+// latency with the slope kernel overlapped, against gemv_kernel with its tail: ELT SH
+// (5316 x 8608) 40.5 -> 35.5 and 41.2 -> 36.6 us, ELT pyramid 50.8 -> 47.7 and 52.0 ->
+// 45.0 us, MCAO 243.2 -> 242.3 and 251.2 -> 250.9 us; with the tail: 42.6, 50.8, 247.5 us;
+// nine vectors in flight 37.4, 49.8, 248.4 us; six CTAs 35.5, 47.7, 244.3 us.  LTAO
+// float32 with its POLC product on it too, frame period 155.2 -> 152.8 us.
+// A row chunk's block stays with gemv_kernel_1row: two cameras' chunks 87.3 us against
+// 90.8 us with this kernel (its registers leave the other camera's slopes less room),
+// although one camera's gain (2500 x 8608 in 8 chunks 69.5 -> 65.2 us).
+constexpr int kWideU = 8, kWideCtas = 5;
 template <int RPW>
-__global__ void __launch_bounds__(kGemvWarps * 32, 5) gemv_kernel_wide(const __grid_constant__ GemvArgs a) {
+__global__ void __launch_bounds__(kGemvWarps * 32, kWideCtas) gemv_kernel_wide(const __grid_constant__ GemvArgs a) {
     gemv_body<RTC_F32, kWideU, 1, RPW, false, 1, false, false>(a);
 }
 
@@ -1146,7 +1151,7 @@ cudaError_t launch_gemv_t(const GemvArgs& base, int nb, long long avg_row_bytes,
     const dim3 grid = fill(rpw, 1);
     // rows of more vectors than the other float32 kernels keep in flight (4 x 32 of 16 bytes)
     if constexpr (DT == RTC_F32 && !kG)
-        if (a.whole && avg_row_bytes > 2048)
+        if (avg_row_bytes > 2048 && (a.whole || (!a.fin.enabled && rpw == 1 && grid.x <= kWideCtas * 152)))
             return launch_maybe_pdl(rpw >= 4 ? gemv_kernel_wide<4> : gemv_kernel_wide<1>, grid, a, pdl, st);
     if (rpw >= 4) return launch_maybe_pdl(gemv_kernel<DT, U, RI, (RI > 4 ? RI : 4), kG, 1>, grid, a, pdl, st);
     if constexpr (!kNoRpw2)
