@@ -36,21 +36,24 @@ struct WfsDev {
 
 // One slope row: a subaperture row (SH) or a pupil row (pyramid).
 struct SlopeRow {
-    int wfs;
+    uint16_t wfs;
+    uint16_t nparts;          // CTAs sharing this row (split by pixel rows)
+    uint16_t x0, x1;          // its first to last valid units: unit columns [x0, x1), empty without any
     int row;                  // row index within its WFS
     int unit0;                // first entry of this row in the unit x-list
     int nunits;               // valid units in this row
     int s_pad;                // padded slope-buffer index of the row's first slope
     int s_compact;            // compact slope index of the row's first slope
-    int nparts;               // CTAs sharing this row (split by pixel rows)
     int pscr;                 // float offset of this row's per-part sums (nparts > 1)
 };
 
-// One CTA of the slope kernel: pixel rows [pr0, pr1) of a subaperture row.
+// One CTA of the slope kernel: some pixel rows of a subaperture row.
 struct SlopePart {
     int row;                  // slope-row table index
-    int part;                 // part index within the row
-    int pr0, pr1;             // pixel rows within the subaperture (SH); unused for pyramid rows
+    uint16_t part;            // part index within the row
+    uint16_t pr0, nrows;      // pixel rows [pr0, pr0 + nrows) of the subaperture (SH); unused for pyramid rows
+    uint16_t gap0, gap1;      // widest run of unit columns [gap0, gap1) without a valid unit inside [x0, x1) (SH)
+    uint16_t pad;
 };
 
 // Everything one slope-kernel CTA needs from the plan, read with one set of

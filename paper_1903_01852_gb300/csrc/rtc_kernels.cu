@@ -92,7 +92,7 @@ __device__ __forceinline__ void store_pair(float* __restrict__ s_pad, int pad, c
     store_pair_v(s_pad, pad, ref != nullptr, load_pair(ref, comp), pol != nullptr, load_pair(pol, comp), sx, sy);
 }
 
-// SH slope-row part: pixel rows [pr0, pr1) of one subaperture row.  The CTA
+// SH slope-row part: some pixel rows of one subaperture row.  The CTA
 // first reduces each pixel column of the strip over its rows (column flux F_c
 // and first moment in y), in G row groups so that narrow strips still use the
 // whole CTA, four rows of loads in flight per thread; then each valid
@@ -123,7 +123,7 @@ __device__ void sh_part(const SlopePart& P, const SlopeRow& row, const WfsDev& W
     const int y0 = W.oy + row.row * n;
     const int q0 = x0 >> 2;                     // quads of 4 pixels aligned to absolute columns
     const int nq = ((x0 + ws + 3) >> 2) - q0;
-    const int nr = P.pr1 - P.pr0;
+    const int nr = P.nrows, pr1 = P.pr0 + nr;
     const int G = max(1, min(nr, (int)blockDim.x / nq));
     float* colF = sm;                           // [G][ws]
     float* colY = sm + G * ws;                  // [G][ws]
@@ -143,10 +143,19 @@ __device__ void sh_part(const SlopePart& P, const SlopeRow& row, const WfsDev& W
         }
     }
 
-    for (int idx = threadIdx.x; idx < nq * G; idx += blockDim.x) {
-        const int q = idx % nq;
-        const int g = idx / nq;
-        const int xa = (q0 + q) << 2;
+    // only the quads of the row's first to last valid subaperture, without those inside
+    // its widest gap: an annular pupil leaves out a third of the strips' pixels.  Frames in
+    // page-locked memory are bound by the link (186 GB/s, whatever the loads): six 68 x 68
+    // sensors, 41.4 -> 32.3 us; in HBM latency bounds it (MCAO 14.9 -> 14.5 us hot, 20.0 ->
+    // 17.8 us from cold caches).
+    const int qlo = (x0 + row.x0 * n) >> 2;
+    const int skip0 = ((x0 + P.gap0 * n + 3) >> 2) - qlo;
+    const int skip = max(0, ((x0 + P.gap1 * n) >> 2) - qlo - skip0);
+    const int nv = row.x1 > row.x0 ? ((x0 + row.x1 * n + 3) >> 2) - qlo - skip : 0;
+    for (int idx = threadIdx.x; idx < nv * G; idx += blockDim.x) {
+        const int q = idx % nv;
+        const int g = idx / nv;
+        const int xa = (qlo + q + (q >= skip0 ? skip : 0)) << 2;
         float F[4] = {0.f, 0.f, 0.f, 0.f};
         float Y[4] = {0.f, 0.f, 0.f, 0.f};
         int r = P.pr0 + g;
@@ -157,7 +166,7 @@ __device__ void sh_part(const SlopePart& P, const SlopeRow& row, const WfsDev& W
 #pragma unroll
             for (int j = 0; j < kRowsInFlight; ++j) {
                 const int rr = r + j * G;
-                if (rr < P.pr1) {
+                if (rr < pr1) {
                     const long long yy = y0 + rr;
                     rw[j] = __ldg(reinterpret_cast<const uint2*>(px + (yy - prow0) * pitch + xa));
                     d[j] = __ldg(reinterpret_cast<const float4*>(W.dark + yy * W.calib_pitch + xa));
@@ -167,7 +176,7 @@ __device__ void sh_part(const SlopePart& P, const SlopeRow& row, const WfsDev& W
 #pragma unroll
             for (int j = 0; j < kRowsInFlight; ++j) {
                 const int rr = r + j * G;
-                if (rr < P.pr1) {
+                if (rr < pr1) {
                     const uint2 q2 = rw[j];
                     const float yc = float(rr) - half;
                     const float t0 = calibrate(q2.x & 0xffffu, d[j].x, f[j].x, T, mode);
@@ -181,7 +190,7 @@ __device__ void sh_part(const SlopePart& P, const SlopeRow& row, const WfsDev& W
             }
             r += kRowsInFlight * G;    // rows beyond (never with the default part split) go below
         }
-        for (; r + 3 * G < P.pr1; r += 4 * G) {
+        for (; r + 3 * G < pr1; r += 4 * G) {
             uint2 rw[4];
             float4 d[4], f[4];
 #pragma unroll
@@ -203,7 +212,7 @@ __device__ void sh_part(const SlopePart& P, const SlopeRow& row, const WfsDev& W
                 Y[2] = fmaf(t2, yc, Y[2]); Y[3] = fmaf(t3, yc, Y[3]);
             }
         }
-        for (; r < P.pr1; r += G) {
+        for (; r < pr1; r += G) {
             const long long yy = y0 + r;
             const uint2 rw = __ldg(reinterpret_cast<const uint2*>(px + (yy - prow0) * pitch + xa));
             const float4 d = __ldg(reinterpret_cast<const float4*>(W.dark + yy * W.calib_pitch + xa));
@@ -405,7 +414,7 @@ __global__ void __launch_bounds__(32) chunk_gate_kernel(const ChunkGate g) {
 }
 
 template <bool kAllRows, bool kGated>
-__global__ void __launch_bounds__(kSlopeThreads) slopes_kernel(const __grid_constant__ SlopeArgs a) {
+__global__ void __launch_bounds__(kSlopeThreads, kAllRows ? 1 : 4) slopes_kernel(const __grid_constant__ SlopeArgs a) {
     extern __shared__ float sm[];
     __shared__ ChunkDesc s_box;
     if constexpr (kGated) {

@@ -550,7 +550,9 @@ int create_impl(const rtc_geometry* G, const rtc_calib* C, const rtc_cmat* M, co
             int local = 0;
             for (int i = r0; i < r1; ++i) {
                 SlopeRow R{};
-                R.wfs = k;
+                R.wfs = (uint16_t)k;
+                R.x0 = row_x[i].empty() ? 0 : row_x[i].front();
+                R.x1 = row_x[i].empty() ? 0 : (uint16_t)(row_x[i].back() + 1);
                 R.row = i;
                 R.unit0 = (int)xlist.size();
                 R.nunits = (int)row_x[i].size();
@@ -600,7 +602,6 @@ int create_impl(const rtc_geometry* G, const rtc_calib* C, const rtc_cmat* M, co
             const int nq = ((w.ox + ws + 3) >> 2) - (w.ox >> 2);
             D.sh_groups = std::max(1, std::min(w.npx, kSlopeThreads / nq));
             L->smem_bytes = std::max(L->smem_bytes, (int)(2 * D.sh_groups * ws * sizeof(float)));
-            L->pixel_bytes += (size_t)w.nsuby * w.npx * (size_t)nq * 4 * (2 + 8);
         }
     }
     // pyramid pixel bytes: 4 pixels x (2 + 8) bytes per valid unit
@@ -626,17 +627,26 @@ int create_impl(const rtc_geometry* G, const rtc_calib* C, const rtc_cmat* M, co
             const int rpt = RTC_SLOPE_ROWS_PER_THREAD;
             np = std::min(w.npx, std::max(1, (w.npx + rpt * gfull - 1) / (rpt * gfull)));
         }
-        R.nparts = np;
+        R.nparts = (uint16_t)np;
         R.pscr = (int)pscr_floats;
         if (np > 1) pscr_floats += (size_t)np * R.nunits * 3;
         L->part_start.push_back((int)parts.size());
         for (int k = 0; k < np; ++k) {
             SlopePart P{};
             P.row = r;
-            P.part = k;
-            P.pr0 = w.kind == RTC_WFS_SH ? (k * w.npx) / np : 0;
-            P.pr1 = w.kind == RTC_WFS_SH ? ((k + 1) * w.npx) / np : 0;
+            P.part = (uint16_t)k;
+            P.pr0 = (uint16_t)(w.kind == RTC_WFS_SH ? ((long long)k * w.npx) / np : 0);
+            P.nrows = (uint16_t)(w.kind == RTC_WFS_SH ? (int)(((long long)(k + 1) * w.npx) / np) - P.pr0 : 0);
+            for (int u = 1; w.kind == RTC_WFS_SH && u < R.nunits; ++u) {
+                const int a = xlist[R.unit0 + u - 1] + 1, b = xlist[R.unit0 + u];
+                if (b - a > P.gap1 - P.gap0) { P.gap0 = (uint16_t)a; P.gap1 = (uint16_t)b; }
+            }
             parts.push_back(P);
+            if (k == 0 && R.x1 > R.x0) {     // the quads of 4 pixels that the slope kernel reads of the row's strip
+                const int skip = std::max(0, ((w.ox + P.gap1 * w.npx) >> 2) - ((w.ox + P.gap0 * w.npx + 3) >> 2));
+                const int nv = ((w.ox + R.x1 * w.npx + 3) >> 2) - ((w.ox + R.x0 * w.npx) >> 2) - skip;
+                if (w.kind == RTC_WFS_SH) L->pixel_bytes += (size_t)w.npx * (size_t)nv * 4 * (2 + 8);
+            }
         }
     }
     L->part_start.push_back((int)parts.size());
