@@ -701,7 +701,7 @@ def ours_arm(args, world, rank, local):
         "roofline": {"bound": "hbm", "achieved": gbs["f32"], "peak": peak, "unit": "GB/s",
                      "frac": gbs["f32"] / peak, "traffic": traffic, "kernel": "gemv_kernel<f32> (reconstruction MVM)",
                      "algorithmic_bytes_per_launch": mb, "peak_kind": peak_kind},
-        "gpu_launches": 4 * args.steps,   # per frame: slopes, MVM (with finalisation), telemetry pack, POLC
+        "gpu_launches": 5 * args.steps,   # per frame: slopes, MVM, finalisation, telemetry pack, POLC
         "clocks": sampler.summary(),
     }
     if cpu:

@@ -207,7 +207,8 @@ cudaError_t launch_slopes(const SlopeCta* ctas, int cta0, int nctas, const WfsDe
 // GEMV over blocks [b0, b0 + nb): out[b * out_stride + r] = sum_j M_b[r][j] x[x_off_b + j],
 // times out_scale[r] when out_scale is not NULL; with fin, the CTA completing the
 // last block of a row tile also finalises it (a, cmd) and the last tile sets the
-// completion word.  pdl: launched as a programmatic dependent of the previous
+// completion word (a large launch of all a frame's blocks leaves that to a kernel
+// launched after it).  pdl: launched as a programmatic dependent of the previous
 // kernel in the stream (prefetches matrix tiles into L2, then waits for it);
 // avg_row_bytes sizes that prefetch.  gate_state: a pre-enqueued chunk's settled
 // mailbox state (device memory), read after that wait; the launch does nothing

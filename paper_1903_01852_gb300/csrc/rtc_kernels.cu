@@ -8,10 +8,14 @@
 //                    is memory-bandwidth bound), with the finalisation (partial
 //                    sums + POLC term + leaky integrator, Section 3 and 3.4)
 //                    fused into its tail; also the POLC product P a (or D a in
-//                    explicit-POLC mode)
+//                    explicit-POLC mode).  _grouped: several column blocks per
+//                    CTA, _deep: few CTAs of a narrow format, _wide: long float32
+//                    rows, _1row: small float32 launches
+//   finalise_kernel  the finalisation of a large whole frame
 //   normalise_kernel global normalisation of pyramid slopes by the mean flux
 //   telemetry_kernel one entry of the telemetry circular buffer (Section 3.3)
-//   pack / relayout / quantize / check kernels used at creation and for telemetry
+//   pack / relayout / lane order / quantize / check kernels used at creation and for
+//                    telemetry
 #include <algorithm>
 #include <type_traits>
 
@@ -582,8 +586,9 @@ cudaError_t launch_slopes(const SlopeCta* ctas, int cta0, int nctas, const WfsDe
 // GEMV: one warp per matrix row of a column block.  Each lane streams 16-byte
 // vectors v = lane, lane+32, ... of the row (U of them in flight), multiplies
 // by the matching input elements (read-only cache) and accumulates in float32;
-// a fixed xor-butterfly reduces the 32 lane sums.  The order of every sum is
-// fixed, so a block's partial does not depend on how the launch was split.
+// a fixed xor-butterfly reduces the lane sums (E4M3: 16 lanes to a row, two rows a
+// warp).  The order of every sum is fixed, so a block's partial does not depend on how
+// the launch was split or which of the kernels below took it.
 // ---------------------------------------------------------------------------
 // Lanes to a row of an E4M3 matrix.  A block's row is short (MCAO: 69 vectors of 16
 // bytes), so 32 lanes leave its last step mostly empty (5 of 32 lanes); 16 lanes waste
@@ -617,9 +622,10 @@ __device__ __forceinline__ float bf_hi(uint32_t u) { return __uint_as_float(u & 
 // Consecutive column blocks one MVM CTA takes (its row tile of each, one fused
 // finalisation for all), per storage format.  BF16 and E4M3 rows of a block are
 // short (about 2.2 and 1.1 KB on MCAO), so a one-block CTA spends much of its
-// life on its fixed costs; two blocks per CTA: MCAO BF16 MVM 138.9 -> 132.7 us,
-// E4M3 108.1 -> 99.9 us, LTAO BF16 85.6 -> 75.4 us.  Float32 rows are long
-// enough (one block: 243.2 us, two: 245.3 us).
+// life on its fixed costs; one / two blocks per CTA: E4M3 MVM, MCAO 86.6 / 80.4 us,
+// LTAO 55.9 / 51.7 us, BF16, LTAO 78.4 / 74.2 us, MCAO 129.6 us with both (with three
+// the frame period is the same).  Float32 rows are long enough (one block: 243.2 us,
+// two: 245.3 us).
 #ifndef RTC_GEMV_GROUP_F32
 #define RTC_GEMV_GROUP_F32 1
 #endif
@@ -868,7 +874,7 @@ __device__ __forceinline__ void gemv_body(const GemvArgs& a) {
         }
     }
     pdl_wait();           // the input vector (slopes or commands) is written by the previous kernel
-    pdl_trigger();
+    pdl_trigger();        // after the wait: slope kernels launched beside this one count on what it waited for
     if constexpr (kGated)     // written by the gate kernel, ahead of the slope kernel waited for above
         if (__ldcg(a.gate_state) != kChunkFilled) return;
 #pragma unroll 1
@@ -1112,9 +1118,9 @@ cudaError_t launch_maybe_pdl(K kernel, dim3 grid, const GemvArgs& a, bool pdl, c
 
 // Launches too small for RTC_GEMV_MIN_WAVES waves of 8 CTAs per SM at four rows
 // per warp take fewer rows per warp.  Two waves: the ELT SCAO MVM (5316 x 8608,
-// 8 blocks) runs one row per warp in 5344 CTAs, and more of them start while the
-// slope kernel runs and prefetch their tiles into L2 (frame latency 43.3 against
-// 45.1 us with one wave, although the MVM alone is slower: 40.6 against 36.5 us).
+// 8 blocks) runs one row per warp in 5320 CTAs, and more of them start while the
+// slope kernel runs and prefetch their tiles into L2 (frame latency 36.6 against
+// 43.2 us with one wave, MVM alone 35.5 against 37.5 us).
 #ifndef RTC_GEMV_MIN_WAVES
 #define RTC_GEMV_MIN_WAVES 2
 #endif

@@ -1417,7 +1417,7 @@ int submit_impl(rtc_loop* L, const rtc_chunk* c) {
 
 // Stream work of one whole frame whose pixels are addressed by fp: slopes of
 // every row, the MVM (a programmatic dependent of the slope kernel) with its
-// fused finalisation, then the tail.  Shared by rtc_process_frame and the
+// finalisation, then the tail.  Shared by rtc_process_frame and the
 // captured frame graphs.
 int enqueue_whole_frame(rtc_loop* L, const FramePtrs& fp) {
     Slot& s = L->slots[L->cur_slot];
