@@ -1521,7 +1521,7 @@ int process_impl(rtc_loop* L, uint64_t id, const uint16_t* const* px, const size
     return status;
 }
 
-// CTAs of an update's reordering kernel over the whole matrix, few so that the frames
+// CTAs of an update's reordering kernel (at least one per column block), few so that the frames
 // running meanwhile keep their bandwidth.
 constexpr int kUpdateCtas = 16;
 
