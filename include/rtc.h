@@ -300,8 +300,10 @@ int rtc_submit_pixels_n(rtc_loop* loop, const rtc_chunk* chunks, int32_t n, int3
  * WFS w's frame (16-byte aligned), pitch[w] is its row pitch in bytes (a
  * multiple of 16, >= 2*width rounded up to 16); pageable memory is rejected
  * with RTC_EINVAL.  The slope kernels read the frames in place; they must
- * stay unchanged until rtc_get_commands returns this frame.  Otherwise
- * behaves like submitting every row of every WFS at once. */
+ * stay unchanged until rtc_get_commands returns this frame.  They are complete
+ * at the call, or written by work queued before it on the loop's stream
+ * (rtc_get_stream).  Otherwise behaves like submitting every row of every WFS
+ * at once. */
 int rtc_process_frame(rtc_loop* loop, uint64_t frame_id,
                       const uint16_t* const* px, const size_t* pitch);
 
@@ -459,7 +461,11 @@ int rtc_sync(rtc_loop* loop);
 int rtc_check_guards(rtc_loop* loop, int32_t* corrupted);
 
 /* The loop's CUDA stream (a cudaStream_t) in *stream, so a caller can order
- * its own work or timing events after the loop's; the loop keeps ownership. */
+ * its own work or timing events after the loop's, or whole frames
+ * (rtc_process_frame) after its own work: a kernel queued there may write the
+ * pixels of the next frame.  From this call on, a frame's slopes no longer
+ * start beside the POLC product of the frame before (a frame period of an
+ * implicit-POLC loop is then up to 5 us longer).  The loop keeps ownership. */
 int rtc_get_stream(rtc_loop* loop, void** stream);
 
 typedef struct rtc_info {

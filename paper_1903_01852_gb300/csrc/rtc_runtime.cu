@@ -116,6 +116,7 @@ struct rtc_loop {
     std::vector<Slot> slots;
 
     cudaStream_t st = nullptr, st_tel = nullptr;
+    std::atomic<bool> st_shared{false};      // rtc_get_stream has handed st out: its last kernel may be the caller's
     // per WFS: the stream its chunks' work runs on (cameras overlap on the device), and its join event
     std::vector<cudaStream_t> st_w;
     std::vector<cudaEvent_t> ev_w;
@@ -1431,8 +1432,10 @@ int enqueue_whole_frame(rtc_loop* L, const FramePtrs& fp) {
     // With an implicit POLC the stream's last kernel is the POLC product of the frame before, which lets
     // this frame start once it has waited for that frame's MVM (nothing of this frame but the finalisation
     // reads what it writes): the slopes run beside it.  Frame period, MCAO float32 286.5 -> 281.5 us, BF16
-    // 155.6 -> 153.2, E4M3 106.0 -> 104.4, LTAO E4M3 72.8 -> 71.4.
-    const bool beside = L->has_polc && !L->timing && !L->capturing;
+    // 155.6 -> 153.2, E4M3 106.0 -> 104.4, LTAO E4M3 72.8 -> 71.4.  Not once a caller has the stream: its
+    // last kernel may then be the caller's, which writes these pixels, and the slope kernel does not wait
+    // before it reads them.
+    const bool beside = L->has_polc && !L->timing && !L->capturing && !L->st_shared.load();
     TRY(slopes_rows(L, 0, L->nrows, fp, false, L->st, nullptr, beside));
     if (L->stage_timing) TRY(record(L, s.ev_slopes, L->st));
     const FinaliseArgs fa = fin_args(L);
@@ -2091,6 +2094,7 @@ int rtc_check_guards(rtc_loop* L, int32_t* corrupted) {
 
 int rtc_get_stream(rtc_loop* L, void** stream) {
     if (!L || !stream) return fail(L, RTC_EINVAL, "loop and stream are required");
+    L->st_shared.store(true);
     *stream = static_cast<void*>(L->st);
     return RTC_OK;
 }
