@@ -180,6 +180,7 @@ int create(const rtc_master_desc* d, rtc_master* m) {
             std::memcpy(rowed.data() + r * B.pitch * esz, static_cast<const unsigned char*>(P->P) + r * na * esz,
                         na * esz);
         MCK(m, cudaMemcpyAsync(m->d_P, rowed.data(), m->p_bytes, cudaMemcpyHostToDevice, m->st));
+        MCK(m, cudaStreamSynchronize(m->st));      // the GPU may read pageable memory in place until then
         MCK(m, launch_lane_order(m->p_dtype, m->d_P, m->d_pblock, 1, m->na, B.pitch, 4096, m->st));
         if (P->row_scale) {
             rc = malloc_dev(m, &m->d_pscale, na * 4);
