@@ -1167,7 +1167,8 @@ cudaError_t launch_gemv_t(const GemvArgs& base, int nb, long long avg_row_bytes,
     // rows of more vectors than the other float32 kernels keep in flight (4 x 32 of 16 bytes)
     if constexpr (DT == RTC_F32 && !kG)
         if (avg_row_bytes > 2048 && (a.whole || (!a.fin.enabled && rpw == 1 && grid.x <= kWideCtas * 152)))
-            return launch_maybe_pdl(rpw >= 4 ? gemv_kernel_wide<4> : gemv_kernel_wide<1>, grid, a, pdl, st);
+            return rpw >= 4 ? launch_maybe_pdl(gemv_kernel_wide<4>, grid, a, pdl, st)
+                            : launch_maybe_pdl(gemv_kernel_wide<1>, fill(1, 1), a, pdl, st);
     if (rpw >= 4) return launch_maybe_pdl(gemv_kernel<DT, U, RI, (RI > 4 ? RI : 4), kG, 1>, grid, a, pdl, st);
     if constexpr (!kNoRpw2)
         if (rpw >= 2) return launch_maybe_pdl(gemv_kernel<DT, U, RI, (RI > 2 ? RI : 2), kG, 1>, grid, a, pdl, st);
