@@ -599,6 +599,7 @@ cudaError_t launch_slopes(const SlopeCta* ctas, int cta0, int nctas, const WfsDe
 #define RTC_GEMV_E4M3_LANES 16
 #endif
 constexpr int kLanesE4m3 = RTC_GEMV_E4M3_LANES;
+static_assert(kLanesE4m3 == 16 || kLanesE4m3 == 32, "lanes to a row (the deep kernels work on two rows a warp)");
 
 template <int DT> struct Elem;
 template <> struct Elem<RTC_F32> { static constexpr int kPer16 = 4, kLanes = 32; };
@@ -655,6 +656,12 @@ __device__ __forceinline__ acc_pk fma2(float a0, float a1, float b0, float b1, a
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ float acc_add(float a, float b) { return a + b; }
+__device__ __forceinline__ acc_pk acc_add(acc_pk a, acc_pk b) {
+    acc_pk d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 __device__ __forceinline__ float acc_total(float c) { return c; }
 __device__ __forceinline__ float acc_total(acc_pk c) {
     float lo, hi;
@@ -704,7 +711,7 @@ __device__ __forceinline__ A dot_e4m3(const uint4& m, const float4* x, int w, A 
         sum = fma2(lo.x, lo.y, xv.x, xv.y, sum);
         sum = fma2(hi.x, hi.y, xv.z, xv.w, sum);
     }
-    return acc + sum;
+    return acc_add(acc, sum);
 }
 
 // Lane order: the columns of an E4M3 row that the 16 bytes of a lane hold.  A row is

@@ -48,3 +48,10 @@ def run_with(defines, tmp_path, cases):
 def test_float32_sums_of_one_fma_per_element(tmp_path):
     # without packed sums a launch may take two rows per warp: whole frames of 50000 rows x blocks, rows of 160 vectors
     run_with(["RTC_GEMV_FFMA2_MASK=0"], tmp_path, [("f32", 80, 2500, 20), ("f32", 24, 240, 3)])
+
+
+@pytest.mark.parametrize("lanes", [16, 32])
+def test_packed_sums_of_the_narrow_formats(tmp_path, lanes):
+    # few-CTA launches (four and two rows per warp), grouped whole frames, rows of one vector to 50
+    cases = [(fmt, *size) for fmt in ("e4m3", "bf16") for size in ((24, 200, 3), (6, 33, 5), (40, 2500, 4))]
+    run_with(["RTC_GEMV_FFMA2_MASK=7", f"RTC_GEMV_E4M3_LANES={lanes}"], tmp_path, cases + [("e4m3", 60, 6000, 28)])
