@@ -17,6 +17,7 @@
 //   pack / relayout / lane order / quantize / check kernels used at creation and for
 //                    telemetry
 #include <algorithm>
+#include <cstring>
 #include <type_traits>
 
 #include <cuda_bf16.h>
@@ -1407,8 +1408,8 @@ __global__ void __launch_bounds__(kThreads, kCtas)
         if (aligned) {
             *reinterpret_cast<Four*>(o) = c;
         } else {
-            Code one[4];
-            *reinterpret_cast<Four*>(one) = c;
+            alignas(Four) Code one[4];
+            memcpy(one, &c, sizeof(c));
 #pragma unroll
             for (int k = 0; k < 4; ++k) o[k] = one[k];
         }
