@@ -197,8 +197,15 @@ cudaError_t launch_normalise(const int2* items, int item0, int nitems, int max_p
 // variant that keeps all of a thread's pixel rows in flight, for small launches
 // that read pixels in place from page-locked host memory.  Each slope is
 // (measured - ref) + pol, with ref and pol (compact slope order) optional.  beside:
-// launched as a programmatic dependent of the stream's last kernel, which must be one of
-// the same frame on other slope rows; it starts beside that kernel and ends after it.
+// launched as a programmatic dependent of the stream's last kernel; it starts beside that
+// kernel, without waiting for it, and ends after it.  So that kernel must not write what
+// these slopes read (pixels, ref, pol), and whatever reads or writes what they write
+// (their rows of s_pad, pscr and counters) must have ended before that kernel lets its
+// dependents start.  Two uses: a camera's later chunk of a frame, behind the MVM (or
+// slopes) of the chunk before, which touches other rows; and a whole frame with implicit
+// POLC (pol NULL) behind the POLC product of the frame before, which starts its dependents
+// only after it has waited for that frame's MVM (gemv_body) and, through the loop's
+// stream, for that frame's telemetry.
 cudaError_t launch_slopes(const SlopeCta* ctas, int cta0, int nctas, const WfsDev* wfs, int nwfs,
                           const FramePtrs& fp, bool host_px, const uint16_t* xlist, const float* ref,
                           const float* pol, float* s_pad, float* pscr, unsigned* counters, int smem_bytes,

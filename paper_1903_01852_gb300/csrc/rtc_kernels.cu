@@ -463,8 +463,9 @@ __global__ void __launch_bounds__(kSlopeThreads, kAllRows ? 1 : 4) slopes_kernel
                                   a.counters, sm);
     else
         pyr_row(row, W, px, pitch, prow0, a.xlist, a.ref, a.pol, a.s_pad, a.pscr);
-    // A later chunk's launch runs beside the MVM of the chunk before, but is not complete
-    // before that is: what waits for this kernel has all of the frame's earlier work done.
+    // Launched beside the stream's last kernel (a later chunk beside the MVM of the chunk
+    // before, a whole frame beside the POLC product of the frame before), but not complete
+    // before that is: what waits for this kernel has all of the stream's earlier work done.
     // ELT SH, 8 chunks in page-locked memory, frame period float32 112 -> 72 us, BF16 108
     // -> 64 us, SCAO 16 x 16 in 4 chunks 38 -> 32 us (the register-light variant, which
     // finds room beside more of the MVM's CTAs, takes longer over the link: 98, 92, 31 us).
