@@ -747,7 +747,6 @@ struct GemvArgs {
     int prefetch_ctas;         // CTAs [0, prefetch_ctas) prefetch their matrix tile into L2 before waiting
     const int* gate_state;     // a pre-enqueued chunk's mailbox state: unless kChunkFilled, do nothing
     bool whole;                // the MVM of a whole frame, finalised by a kernel of its own
-    int group;                 // column blocks per CTA (consecutive, same row tile), >= 1
 };
 
 #ifndef RTC_GEMV_F32_U
@@ -1147,10 +1146,9 @@ cudaError_t launch_gemv_t(const GemvArgs& base, int nb, long long avg_row_bytes,
     constexpr bool kNoRpw2 = RI == 1 && std::is_same<typename AccOf<DT>::type, acc_pk>::value;
     if (kNoRpw2 && rpw == 2) rpw = 1;
     GemvArgs a = base;
-    a.tiles = (na + kGemvWarps * rpw - 1) / (kGemvWarps * rpw);
+    const int tiles = (na + kGemvWarps * rpw - 1) / (kGemvWarps * rpw);
     const auto fill = [&](int rows, int group) {            // the grid, and the prefetch of its first tiles
         a.tiles = (na + kGemvWarps * rows - 1) / (kGemvWarps * rows);
-        a.group = group;
         const dim3 grid((unsigned)(a.tiles * ((nb + group - 1) / group)));
         // prefetch while waiting for the producer: about 96 MB, below the L2 size
         const long long tile_bytes = std::max(1LL, avg_row_bytes * kGemvWarps * rows * group);
@@ -1160,12 +1158,12 @@ cudaError_t launch_gemv_t(const GemvArgs& base, int nb, long long avg_row_bytes,
     // consecutive column blocks per CTA, if that keeps enough CTAs
     constexpr int kMaxGroup = DT == RTC_F32 ? RTC_GEMV_GROUP_F32 : DT == RTC_BF16 ? RTC_GEMV_GROUP_BF16 : RTC_GEMV_GROUP_E4M3;
     if constexpr (kMaxGroup > 1)
-        if (rpw >= 4 && (long long)a.tiles * ((nb + kMaxGroup - 1) / kMaxGroup) >= RTC_GEMV_GROUP_MIN_WAVES * 8LL * 152)
+        if (rpw >= 4 && (long long)tiles * ((nb + kMaxGroup - 1) / kMaxGroup) >= RTC_GEMV_GROUP_MIN_WAVES * 8LL * 152)
             return launch_maybe_pdl(gemv_kernel_grouped<DT, U, RI, (RI > 4 ? RI : 4), kG, kMaxGroup>, fill(rpw, kMaxGroup), a,
                                     pdl, st);
     // few CTAs: deep kernels (see Deep)
     if constexpr (DT != RTC_F32 && RI == 4) {
-        const long long ctas = (long long)a.tiles * nb;
+        const long long ctas = (long long)tiles * nb;
         if (rpw == RI && ctas <= Deep<DT>::kMaxCtas * (avg_row_bytes >= 2048 ? Deep<DT>::kLongRowFactor : 1)) {
             constexpr int kU = Deep<DT>::kU;
             if (ctas <= 152) return launch_maybe_pdl(gemv_kernel_deep<DT, kU, 2, kG>, fill(2, 1), a, pdl, st);
@@ -1221,7 +1219,7 @@ cudaError_t launch_gemv(int dtype, const void* M, const BlockDev* blocks, int b0
                         long long avg_row_bytes, bool pdl, cudaStream_t st, const int* gate_state) {
     if (nb <= 0 || na <= 0) return cudaSuccess;
     GemvArgs a{static_cast<const uint8_t*>(M), blocks, b0, nb, 0, na, x, out_scale, out, out_stride, FinaliseArgs{}, 0,
-               gate_state, false, 1};
+               gate_state, false};
     if (fin) a.fin = *fin;
     if (fin && fin->enabled && nb == fin->nblk && !gate_state &&
         avg_row_bytes * na * nb >= (dtype == RTC_F32 ? kSeparateMinF32 : kSeparateMinNarrow)) {
