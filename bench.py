@@ -205,7 +205,7 @@ def bf16_config(cfg, rtc, torch):
 
 
 def mvm_bytes(info, cfg):
-    """Algorithmic bytes of one reconstruction MVM launch with its fused finalisation:
+    """Algorithmic bytes of one reconstruction MVM launch with its finalisation:
     matrix (true size) and row scales, the slopes read, the per-block partial commands
     written and read back, and q, a (read and write) and the commands written."""
     b = {"f32": 4, "bf16": 2, "e4m3": 1}[cfg.get("M_dtype", "f32")]
@@ -699,7 +699,7 @@ def ours_arm(args, world, rank, local):
                 "latency_us": stats(e2e_lat), "process_frame_latency_us": stats(pf_lat)},
         "serving_mix": mix,
         "roofline": {"bound": "hbm", "achieved": gbs["f32"], "peak": peak, "unit": "GB/s",
-                     "frac": gbs["f32"] / peak, "traffic": traffic, "kernel": "gemv_kernel<f32> (reconstruction MVM)",
+                     "frac": gbs["f32"] / peak, "traffic": traffic, "kernel": "gemv_kernel_wide<4> (reconstruction MVM)",
                      "algorithmic_bytes_per_launch": mb, "peak_kind": peak_kind},
         "gpu_launches": 5 * args.steps,   # per frame: slopes, MVM, finalisation, telemetry pack, POLC
         "clocks": sampler.summary(),

@@ -316,8 +316,8 @@ int rtc_next_frame_buffers(rtc_loop* loop, uint16_t** px, size_t* pitch);
 
 /* Graph mode: launch the CUDA graph captured at creation for the buffers the
  * last rtc_next_frame_buffers returned (slopes, MVM with finalisation, POLC,
- * telemetry: one launch instead of four kernels and their events).  Frame-id
- * rules as rtc_process_frame. */
+ * telemetry: one launch instead of four or five kernels and their events).
+ * Frame-id rules as rtc_process_frame. */
 int rtc_submit_frame_graph(rtc_loop* loop, uint64_t frame_id);
 
 /* The DM commands of a frame (Section 3: the master's sum of the partial
@@ -338,13 +338,15 @@ int rtc_get_telemetry(rtc_loop* loop, uint64_t frame_id, float* slopes, size_t n
                       float* cmds, size_t na, int64_t timeout_us);
 
 /* Device times of one frame (the latency of Table ao_results, measured on the
- * GPU), from CUDA events on the loop's stream (needs RTC_FLAG_TIMING).  latency_us: for rtc_process_frame, from just before the
- * slope kernel to the end of the MVM kernel, whose tail writes the commands;
- * for chunked frames, from just before the last chunk's work.  frame_us: from
- * the frame's first submitted work to the commands.  polc_us: the POLC
- * product after the commands.  slopes_us and mvm_us (the MVM kernel with its
- * fused finalisation) need RTC_FLAG_STAGE_TIMING, else they are -1;
- * final_us is 0 (the finalisation is part of the MVM kernel).  In graph mode
+ * GPU), from CUDA events on the loop's stream (needs RTC_FLAG_TIMING).
+ * latency_us: for rtc_process_frame, from just before the slope kernel to the
+ * end of the kernel that writes the commands (the MVM, or for a large whole
+ * frame the finalisation kernel behind it); for chunked frames, from just
+ * before the last chunk's work.  frame_us: from the frame's first submitted
+ * work to the commands.  polc_us: the POLC product after the commands.
+ * slopes_us and mvm_us (the MVM with the finalisation, fused or a kernel of
+ * its own) need RTC_FLAG_STAGE_TIMING, else they are -1; final_us is 0 (the
+ * finalisation's time is part of mvm_us).  In graph mode
  * (RTC_FLAG_GRAPHS) latency_us and frame_us span the whole graph launch, POLC
  * and telemetry included, and polc_us is about 0; RTC_FLAG_STAGE_TIMING is not
  * available there. */

@@ -233,8 +233,8 @@ cudaError_t launch_pack_slopes(const BlockDev* blocks, int nblk, int max_cols,
 cudaError_t launch_relayout(int dtype, const void* src, int na, int ns, const BlockDev* blocks,
                             int nblk, int max_pitch, void* dst, cudaStream_t st);
 
-// A narrow matrix in column blocks, row-major, into the order that launch_gemv reads (in
-// place; nothing to do for float32), with at most max_ctas CTAs per column block.
+// An E4M3 matrix in column blocks, row-major, into the order that launch_gemv reads (in
+// place; nothing to do for float32 and BF16), with at most max_ctas CTAs per column block.
 cudaError_t launch_lane_order(int dtype, void* M, const BlockDev* blocks, int nblk, int rows, int max_pitch,
                               int max_ctas, cudaStream_t st);
 

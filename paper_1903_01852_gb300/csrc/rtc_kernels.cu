@@ -111,7 +111,7 @@ __device__ __forceinline__ void store_pair(float* __restrict__ s_pad, int pad, c
 // several times that of HBM): a thread first issues the loads of all its pixel
 // rows (up to kRowsInFlight) and of their dark and flat maps, then calibrates
 // them; the additions keep the same order, so the slopes are bit-identical to the
-// other variant.  It takes ~220 registers (one CTA per SM): right for a chunk's
+// other variant.  It takes 230 registers (one CTA per SM): right for a chunk's
 // few dozen CTAs, not for a whole frame's hundreds.  (Calibration loads in three
 // dependent batches of four rows instead: paced latency 1-2 us longer.)
 constexpr int kRowsInFlight = 12;
@@ -1007,8 +1007,8 @@ __global__ void __launch_bounds__(kGemvWarps * 32, 2) gemv_kernel_deep(const __g
 // (334) 34.8 / 32.8; but rows of 1 KB, 74/8/2000 (504) 26.6 / 27.3.
 // BF16: 71/1/1065 34.7 / 27.2 (29.3), 42/1/1539 25.9 / 23.5, 74/1/5316 39.4 / 36.1,
 // 74/8/1000 25.7 / 25.3, but 74/2/5316 33.9 / 36.1, 74/8/2000 26.9 / 28.0.
-// POLC products: BF16 MCAO (235 CTAs) 24.5 / 22.5 us, LTAO (167) 18.3 / 16.2; E4M3 26.6 /
-// 16.3 and 20.4 / 13.2.
+// POLC products: BF16 MCAO (235 CTAs) 24.5 / 22.5 us, LTAO (167) 18.3 / 14.2; E4M3 26.6 /
+// 16.3 and 20.4 / 12.2.
 template <int DT> struct Deep { static constexpr int kU = 3, kMaxCtas = 304, kLongRowFactor = 1; };
 template <> struct Deep<RTC_E4M3> { static constexpr int kU = 2, kMaxCtas = 304, kLongRowFactor = 2; };
 
